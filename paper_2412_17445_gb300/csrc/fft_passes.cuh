@@ -382,22 +382,24 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? XFWD_MIN_BLOCKS_F32 : 1)
   const int n = (int)g.n;
   const int row0 = blockIdx.x * 2 * P;
   const FDiv dnx = make_fdiv(nx);
-  const double xE = *a.xE_ptr * (a.ks ? a.ks->escale : a.e_scale);
+  T xE;
+  if (sizeof(T) == 4 && a.xEf_ptr) xE = (T)*a.xEf_ptr;
+  else xE = (T)(*a.xE_ptr * (a.ks ? a.ks->escale : a.e_scale));
   T fx[M];
 #pragma unroll
-  for (int k = 0; k < M; ++k) fx[k] = (T)a.fM[k] * (T)xE;
+  for (int k = 0; k < M; ++k) fx[k] = a.fM[k] * xE;
   T beta = 0, omega = 0, alpha = 0;
   bool pending = false;
   if (pm == 1) {
-    beta = (T)a.ks->beta;
-    omega = (T)a.ks->omega;
+    beta = ks_scalar<T>(a.ks->beta, a.ks->beta_f);
+    omega = ks_scalar<T>(a.ks->omega, a.ks->omega_f);
   } else if (pm == 5) {
-    beta = (T)a.ks->beta;
-    omega = (T)a.ks->omega;
-    alpha = (T)a.ks->alpha;
+    beta = ks_scalar<T>(a.ks->beta, a.ks->beta_f);
+    omega = ks_scalar<T>(a.ks->omega, a.ks->omega_f);
+    alpha = ks_scalar<T>(a.ks->alpha, a.ks->alpha_f);
     pending = a.ks->pending != 0;
   } else if (pm == 2) {
-    alpha = (T)a.ks->alpha;
+    alpha = ks_scalar<T>(a.ks->alpha, a.ks->alpha_f);
   }
   // per-thread and warp sums stay in T (a few dozen terms); the block and grid sums are float64
   T wdp = 0;
@@ -559,9 +561,9 @@ __global__ void __launch_bounds__(256) k_xinv_apply(const __grid_constant__ Appl
       else if (a.fin == 5) fin_alpha_clear<true>(a.ksw, a.part, gridDim.x);
       else fin_omega_conv<true>(a.ksw, a.part, gridDim.x);
     }
-  } else if (a.fin == 3 && blockIdx.x == 0) {
+  } else if (a.fin == 3 && blockIdx.x == 0 && threadIdx.x < 32) {
     // the constraint-row partials come from the x-forward pass (an earlier launch)
-    const double sE = sum_partials_t<false>(a.part, gridDim.x);
+    const double sE = warp_sum_exact<false>(a.part, gridDim.x);
     if (threadIdx.x == 0) *a.yE = sE;
   } else if (a.fin == 4 && blockIdx.x == 0 && threadIdx.x == 0) {
     *a.yE = *a.xE_ptr;

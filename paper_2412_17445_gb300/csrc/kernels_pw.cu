@@ -353,39 +353,33 @@ __global__ void __launch_bounds__(256) k_constitutive(ConstArgs a, TK *tan) {
 }
 
 // =========================== reductions ======================================================
-// Deterministic fixed-order sum of G partials (one block, any G), krylov_fin.cuh.
-__device__ double sum_partials(const double *p, int G) { return sum_partials_t<false>(p, G); }
-__device__ double max_partials(const double *p, int G) {
-  __shared__ double red[256];
+// Every quantity by one warp: exact sums (krylov_fin.cuh) or maxima.
+__device__ __forceinline__ double warp_reduce_partials(const double *p, int G, int is_max) {
+  if (!is_max) return warp_sum_exact<false>(p, G);
   double s = -1e308;
-  for (int i = threadIdx.x; i < G; i += blockDim.x) s = fmax(s, p[i]);
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-    if (threadIdx.x < o) red[threadIdx.x] = fmax(red[threadIdx.x], red[threadIdx.x + o]);
-    __syncthreads();
-  }
-  const double r = red[0];
-  __syncthreads();
-  return r;
+  for (int i = threadIdx.x & 31; i < G; i += 32) s = fmax(s, p[i]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s = fmax(s, __shfl_xor_sync(0xffffffffu, s, o));
+  return s;
 }
 
-// out[q] = sum (or max if is_max) of part[q * G .. q * G + G), q < NQ.  <<<1, 256>>>
+// out[q] = sum (or max if is_max) of part[q * G .. q * G + G), q < NQ.  One block.
 __global__ void k_reduce(const double *part, int G, int NQ, int is_max, double *out) {
-  for (int q = 0; q < NQ; ++q) {
-    const double r = is_max ? max_partials(part + (size_t)q * G, G) : sum_partials(part + (size_t)q * G, G);
-    if (threadIdx.x == 0) out[q] = r;
+  for (int q = threadIdx.x >> 5; q < NQ; q += blockDim.x >> 5) {
+    const double r = warp_reduce_partials(part + (size_t)q * G, G, is_max);
+    if ((threadIdx.x & 31) == 0) out[q] = r;
   }
 }
 
 __global__ void k_reduce_list(ReduceList L, double *out) {
+  int w = threadIdx.x >> 5;  // quantities are dealt to the warps in order
   for (int i = 0; i < L.n; ++i) {
     const ReduceSeg &sg = L.s[i];
-    for (int q = 0; q < sg.NQ; ++q) {
-      const double *p = sg.part + (size_t)q * sg.G;
-      const double r = sg.is_max ? max_partials(p, sg.G) : sum_partials(p, sg.G);
-      if (threadIdx.x == 0) out[sg.off + q] = r;
+    for (; w < sg.NQ; w += blockDim.x >> 5) {
+      const double r = warp_reduce_partials(sg.part + (size_t)w * sg.G, sg.G, sg.is_max);
+      if ((threadIdx.x & 31) == 0) out[sg.off + w] = r;
     }
+    w -= sg.NQ;
   }
 }
 
@@ -427,7 +421,9 @@ __global__ void k_kinit(KvArgs<TK> a, int seed, int zero_x) {
 // (re)start: p = v = 0, alpha = omega = 1).  len = c * n.
 __global__ void k_kfin_init(KrylovScalars *ks, const double *part, int G, long long len, int seed,
                             int zero_x) {
-  const double d = sum_partials(part, G);
+  double sum[1];
+  block_sums<1, false>(part, G, sum);
+  const double d = sum[0];
   if (threadIdx.x == 0) {
     const double cz = sqrt(ks->rn2 / ((double)len + 1.0));
     const unsigned long long off = (unsigned long long)seed * (unsigned long long)(len + 1);
@@ -440,6 +436,10 @@ __global__ void k_kfin_init(KrylovScalars *ks, const double *part, int G, long l
     if (zero_x) ks->xE = 0.0;
     ks->pE = ks->rE;
     ks->vE = 0.0;
+    ks->beta_f = (float)rho;
+    ks->alpha_f = ks->omega_f = 1.0f;
+    ks->pE_f = (float)(ks->pE * ks->escale);
+    ks->sE_f = 0.0f;
     ks->status = 0;
     ks->done = 0;
     ks->pending = 0;
@@ -490,8 +490,10 @@ __global__ void k_maxabs(long long len, const TK *t, double *part) {
 // restart: rE = bE - (A x)_E, rn2 = |r|^2
 __global__ void k_kfin_resid(KrylovScalars *ks, const double *part_app, int Gx, const double *part_kv,
                              int Gpw) {
-  const double wdp = sum_partials(part_app, Gx);
-  const double rr = sum_partials(part_kv, Gpw);
+  double s1[1], s2[1];
+  block_sums<1, false>(part_app, Gx, s1);
+  block_sums<1, false>(part_kv, Gpw, s2);
+  const double wdp = s1[0], rr = s2[0];
   if (threadIdx.x == 0) {
     const double yE = ks->strain ? ks->xE : ks->s3 * wdp;  // strain control: no E scaling
     ks->rE = ks->bE - yE;
@@ -504,7 +506,7 @@ template <typename TK>
 __global__ void k_kxr(const __grid_constant__ KvGroup<TK> grp) {
   const KvArgs<TK> &a = grp.m[blockIdx.y];
   if (a.ks->done) return;
-  const TK al = (TK)a.ks->alpha, om = (TK)a.ks->omega;
+  const TK al = ks_scalar<TK>(a.ks->alpha, a.ks->alpha_f), om = ks_scalar<TK>(a.ks->omega, a.ks->omega_f);
   TK rr = 0, rhr = 0;  // per-thread and warp sums in TK, block and grid sums in float64
   long long i0 = 0;
   if constexpr (sizeof(TK) == 4) {
@@ -555,7 +557,7 @@ template <typename TK>
 __global__ void k_kx_finish(const __grid_constant__ KvGroup<TK> grp) {
   const KvArgs<TK> &a = grp.m[blockIdx.y];
   if (!a.ks->pending) return;
-  const TK al = (TK)a.ks->alpha, om = (TK)a.ks->omega;
+  const TK al = ks_scalar<TK>(a.ks->alpha, a.ks->alpha_f), om = ks_scalar<TK>(a.ks->omega, a.ks->omega_f);
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < a.len;
        i += (long long)gridDim.x * blockDim.x) {
     const TK s = a.s[i];

@@ -6,39 +6,84 @@
 #pragma once
 #include "rve_kern.cuh"
 
-// Deterministic fixed-order sum of G partials (one block of 256 threads, any G): Neumaier-
-// compensated per-thread sums, then a tree that carries (sum, compensation) pairs and merges
-// two sums with Knuth's TwoSum (exact rounding error of a + b), so the compensation of every
-// partial reaches the result.  CG: the partials were written by other blocks of the running
-// kernel, so they are read past L1 (ld.global.cg).
+// Exact sum of G float64 partials by one warp, rounded once: each value becomes a 128-bit integer
+// in units of 2^-53 ulp of the largest exponent seen (53 mantissa bits, 53 below them, room for
+// 2^20 terms above), and integers add exactly in any order.  A compensated float64 sum needs five
+// operations a value and seven a tree level on a pipe that takes a warp instruction every 16
+// cycles (the block-wide one took 4.2 us a quantity, 33 us of a 512^2 BiCGStab iteration's
+// seven sums); integer adds run at full rate, a warp a quantity.  Non-finite values fall back
+// to a float64 sum, which propagates them.  CG: the partials were written by other blocks of
+// the running kernel, so they are read past L1 (ld.global.cg).
 template <bool CG>
-__device__ __forceinline__ double sum_partials_t(const double *p, int G) {
-  __shared__ double red[256], cmp[256];
-  double s = 0.0, c = 0.0;
-  for (int i = threadIdx.x; i < G; i += blockDim.x) {
-    const double x = CG ? __ldcg(p + i) : p[i];
-    const double t = s + x;
-    if (fabs(s) >= fabs(x)) c += (s - t) + x;
-    else c += (x - t) + s;
-    s = t;
-  }
-  red[threadIdx.x] = s;
-  cmp[threadIdx.x] = c;
-  __syncthreads();
-  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-    if (threadIdx.x < o) {
-      const double a = red[threadIdx.x], b = red[threadIdx.x + o];
-      const double t = a + b;
-      const double bv = t - a;
-      const double err = (a - (t - bv)) + (b - bv);
-      red[threadIdx.x] = t;
-      cmp[threadIdx.x] += cmp[threadIdx.x + o] + err;
+__device__ __forceinline__ double warp_sum_exact(const double *p, int G) {
+  constexpr int U = 8;  // values per lane in flight
+  const int lane = threadIdx.x & 31;
+  __int128 acc = 0;
+  int E = 1;
+  bool finite = true;
+  for (int base = 0; base < G; base += 32 * U) {
+    unsigned long long b[U];
+    int e = 1;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int i = base + 32 * u + lane;
+      b[u] = i < G ? (unsigned long long)__double_as_longlong(CG ? __ldcg(p + i) : p[i]) : 0ull;
     }
-    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < U; ++u) e = max(e, (int)(b[u] >> 52) & 2047);
+    e = __reduce_max_sync(0xffffffffu, e);
+    finite = finite && e < 2047;
+    if (e > E) {
+      acc = e - E < 127 ? acc >> (e - E) : 0;
+      E = e;
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int ex = (int)(b[u] >> 52) & 2047;
+      const unsigned long long m = (b[u] & 0xFFFFFFFFFFFFFull) | (ex ? 1ull << 52 : 0ull);
+      const int sh = E - (ex ? ex : 1);
+      const __int128 t = sh < 106 ? ((__int128)m << 53) >> sh : 0;
+      acc += (b[u] >> 63) ? -t : t;
+    }
   }
-  const double r = red[0] + cmp[0];
+  if (!finite) {
+    double s = 0.0;
+    for (int i = lane; i < G; i += 32) s += CG ? __ldcg(p + i) : p[i];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long lo = __shfl_xor_sync(0xffffffffu, (unsigned long long)acc, o);
+    const long long hi = __shfl_xor_sync(0xffffffffu, (long long)(acc >> 64), o);
+    acc += (__int128)(((unsigned __int128)(unsigned long long)hi << 64) | lo);
+  }
+  if (acc == 0) return 0.0;
+  const bool neg = acc < 0;
+  unsigned __int128 mag = neg ? (unsigned __int128)(-acc) : (unsigned __int128)acc;
+  const unsigned long long top = (unsigned long long)(mag >> 64);
+  const int lz = top ? __clzll(top) : 64 + __clzll((unsigned long long)mag);
+  mag <<= lz;
+  // the leading 64 bits with the rest as a sticky bit, rounded to 53 once
+  const unsigned long long lead = (unsigned long long)(mag >> 64) | ((unsigned long long)mag ? 1ull : 0ull);
+  const double r = scalbn(__ull2double_rn(lead), 64 - lz + E - 1075 - 53);
+  return neg ? -r : r;
+}
+
+// NQ sums of G partials each (quantity q at part + q G), one warp a quantity; every thread of the
+// block receives them.
+template <int NQ, bool CG>
+__device__ __forceinline__ void block_sums(const double *part, int G, double (&out)[NQ]) {
+  __shared__ double res[NQ];
+  for (int q = threadIdx.x >> 5; q < NQ; q += blockDim.x >> 5) {
+    const double s = warp_sum_exact<CG>(part + (size_t)q * G, G);
+    if ((threadIdx.x & 31) == 0) res[q] = s;
+  }
   __syncthreads();
-  return r;
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) out[q] = res[q];
+  __syncthreads();
 }
 
 // Last-block detection over the blocks of one group member (nblocks of them): every block
@@ -62,8 +107,9 @@ __device__ __forceinline__ bool last_block_arrives(unsigned int *ctr, unsigned i
 // part: G partials of sum w dphi, then G of (rhat, v).
 template <bool CG>
 __device__ __forceinline__ void fin_alpha(KrylovScalars *ks, const double *part, int G) {
-  const double wdp = sum_partials_t<CG>(part, G);
-  const double rv = sum_partials_t<CG>(part + G, G);
+  double sum[2];
+  block_sums<2, CG>(part, G, sum);
+  const double wdp = sum[0], rv = sum[1];
   if (threadIdx.x == 0) {
     ks->vE = ks->strain ? ks->pE : ks->s3 * wdp;
     const double rvt = rv + ks->rhE * ks->vE;
@@ -74,6 +120,8 @@ __device__ __forceinline__ void fin_alpha(KrylovScalars *ks, const double *part,
     }
     ks->alpha = ks->rho / rvt;
     ks->sE = ks->rE - ks->alpha * ks->vE;
+    ks->alpha_f = (float)ks->alpha;
+    ks->sE_f = (float)(ks->sE * ks->escale);
   }
 }
 
@@ -89,14 +137,15 @@ __device__ __forceinline__ void fin_alpha_clear(KrylovScalars *ks, const double 
 // part: G partials of sum w dphi, G of (t, s), G of (t, t).
 template <bool CG>
 __device__ __forceinline__ void fin_omega(KrylovScalars *ks, const double *part, int G) {
-  const double wdp = sum_partials_t<CG>(part, G);
-  const double ts = sum_partials_t<CG>(part + G, G);
-  const double tt = sum_partials_t<CG>(part + 2 * G, G);
+  double sum[3];
+  block_sums<3, CG>(part, G, sum);
+  const double wdp = sum[0], ts = sum[1], tt = sum[2];
   if (threadIdx.x == 0) {
     ks->tE = ks->strain ? ks->sE : ks->s3 * wdp;
     const double tst = ts + ks->tE * ks->sE;
     const double ttt = tt + ks->tE * ks->tE;
     ks->omega = ttt > 0.0 ? tst / ttt : 0.0;
+    ks->omega_f = (float)ks->omega;
     ks->xE += ks->alpha * ks->pE + ks->omega * ks->sE;
     ks->rE = ks->sE - ks->omega * ks->tE;
   }
@@ -106,8 +155,9 @@ __device__ __forceinline__ void fin_omega(KrylovScalars *ks, const double *part,
 // beta (rho_{k+1} from the fused dot).  part: G partials of |r|^2, then G of (rhat, r).
 template <bool CG>
 __device__ __forceinline__ void fin_conv(KrylovScalars *ks, const double *part, int G) {
-  const double rr = sum_partials_t<CG>(part, G);
-  const double rhr = sum_partials_t<CG>(part + G, G);
+  double sum[2];
+  block_sums<2, CG>(part, G, sum);
+  const double rr = sum[0], rhr = sum[1];
   if (threadIdx.x == 0) {
     ks->iters += 1;
     const double rn2 = rr + ks->rE * ks->rE;
@@ -136,6 +186,8 @@ __device__ __forceinline__ void fin_conv(KrylovScalars *ks, const double *part, 
     ks->beta = (rho_new / ks->rho) * (ks->alpha / ks->omega);
     ks->rho = rho_new;
     ks->pE = ks->rE + ks->beta * (ks->pE - ks->omega * ks->vE);
+    ks->beta_f = (float)ks->beta;
+    ks->pE_f = (float)(ks->pE * ks->escale);
   }
 }
 
@@ -148,18 +200,16 @@ __device__ __forceinline__ void fin_conv(KrylovScalars *ks, const double *part, 
 // is left pending; the next x-forward pass or the chunk's closing k_kx_finish applies it.
 template <bool CG>
 __device__ __forceinline__ void fin_omega_conv(KrylovScalars *ks, const double *part, int G) {
-  const double wdp = sum_partials_t<CG>(part, G);
-  const double ts = sum_partials_t<CG>(part + G, G);
-  const double tt = sum_partials_t<CG>(part + 2 * G, G);
-  const double rs = sum_partials_t<CG>(part + 3 * G, G);
-  const double rt = sum_partials_t<CG>(part + 4 * G, G);
-  const double ss = sum_partials_t<CG>(part + 5 * G, G);
+  double sum[6];
+  block_sums<6, CG>(part, G, sum);
+  const double wdp = sum[0], ts = sum[1], tt = sum[2], rs = sum[3], rt = sum[4], ss = sum[5];
   if (threadIdx.x == 0) {
     ks->tE = ks->strain ? ks->sE : ks->s3 * wdp;
     const double tst = ts + ks->tE * ks->sE;
     const double ttt = tt + ks->tE * ks->tE;
     const double om = ttt > 0.0 ? tst / ttt : 0.0;
     ks->omega = om;
+    ks->omega_f = (float)om;
     ks->xE += ks->alpha * ks->pE + om * ks->sE;
     ks->rE = ks->sE - om * ks->tE;
     ks->pending = 1;
@@ -192,5 +242,7 @@ __device__ __forceinline__ void fin_omega_conv(KrylovScalars *ks, const double *
     ks->beta = (rho_new / ks->rho) * (ks->alpha / om);
     ks->rho = rho_new;
     ks->pE = ks->rE + ks->beta * (ks->pE - om * ks->vE);
+    ks->beta_f = (float)ks->beta;
+    ks->pE_f = (float)(ks->pE * ks->escale);
   }
 }

@@ -777,7 +777,7 @@ static ApplyArgs<TK> apply_args(rve *h, TK *x, const double *xE_ptr, TK *y, int 
   a.tan = (const TK *)h->tan;
   a.xE_ptr = xE_ptr;
   a.e_scale = (ks != nullptr) ? h->e_scale : 1.0;
-  for (int k = 0; k < 6; ++k) a.fM[k] = h->fM[k];
+  for (int k = 0; k < 6; ++k) a.fM[k] = (TK)h->fM[k];
   a.spec = (cpx<TK> *)h->spec;
   a.part = h->part.app;
   a.pro_mode = pro_mode;
@@ -804,7 +804,7 @@ static int apply_scaled(rve *h, TK *x, const double *xE_ptr, TK *y, int pro_mode
   a.tan = (const TK *)h->tan;
   a.xE_ptr = xE_ptr;
   a.e_scale = (ks != nullptr) ? h->e_scale : 1.0;
-  for (int k = 0; k < 6; ++k) a.fM[k] = h->fM[k];
+  for (int k = 0; k < 6; ++k) a.fM[k] = (TK)h->fM[k];
   a.spec = spec ? spec : (cpx<TK> *)h->spec;
   a.part = part ? part : h->part.app;
   if (yE) {  // the x-inverse pass also writes the E slot of y (no separate reduction launch)
@@ -836,7 +836,7 @@ static int apply_scaled(rve *h, TK *x, const double *xE_ptr, TK *y, int pro_mode
 
 // ---- host <- device reductions -----------------------------------------------------------
 static int reduce_to_host(rve *h, const double *part, int G, int NQ, int is_max, double *out) {
-  k_reduce<<<1, 256, 0, h->stream>>>(part, G, NQ, is_max, h->red);
+  k_reduce<<<1, 32 * NQ, 0, h->stream>>>(part, G, NQ, is_max, h->red);
   h->launches += 1;
   CKL();
   CK(cudaMemcpyAsync(h->red_h, h->red, sizeof(double) * NQ, cudaMemcpyDeviceToHost, h->stream));
@@ -853,7 +853,7 @@ static int reduce_list_to_host(rve *h, ReduceList L, double *out) {
     L.s[i].off = tot;
     tot += L.s[i].NQ;
   }
-  k_reduce_list<<<1, 256, 0, h->stream>>>(L, h->red);
+  k_reduce_list<<<1, 512, 0, h->stream>>>(L, h->red);
   h->launches += 1;
   CKL();
   CK(cudaMemcpyAsync(h->red_h, h->red, sizeof(double) * tot, cudaMemcpyDeviceToHost, h->stream));
@@ -1283,6 +1283,8 @@ static int issue_chunk_n(rve *const *mem, int nm, cudaStream_t st) {
                                 merged ? kv.s : nullptr, m->ks);
     A2.m[i] = apply_args<TK, M>(m, kv.s, &m->ks->sE, kv.t, 2, merged ? 6 : 2, kv.r, kv.v, kv.rhat, kv.s, m->ks);
     // the x-inverse passes (and k_kxr) finalise the scalars in their last block
+    A1.m[i].xEf_ptr = &m->ks->pE_f;
+    A2.m[i].xEf_ptr = &m->ks->sE_f;
     A1.m[i].fin = merged ? 5 : 1;
     A2.m[i].fin = merged ? 6 : 2;
     A1.m[i].xs = kv.x;
@@ -3354,7 +3356,7 @@ extern "C" int rve_apply_device_noalloc(rve_t *h, const void *x, const double *x
     CK(cudaMemcpyAsync(yE, xE, sizeof(double), cudaMemcpyDeviceToDevice, h->stream));
   } else {
     const double *pd = (const double *)((unsigned char *)scratch + kNoAllocSpecBytes);
-    k_reduce<<<1, 256, 0, h->stream>>>(pd, Gx, 1, 0, yE);
+    k_reduce<<<1, 32, 0, h->stream>>>(pd, Gx, 1, 0, yE);
     h->launches += 1;
     CKL();
   }

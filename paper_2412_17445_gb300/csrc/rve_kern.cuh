@@ -81,7 +81,15 @@ struct KrylovScalars {
   int pending;          // float32 chunks: x += alpha p + omega s, r = s - omega t of the last
                         // iteration not applied yet (the next x-forward pass, or the chunk's
                         // closing k_kx_finish, applies it)
+  // float32 copies for the kernels of a float32 solve, whose threads would otherwise each convert
+  // on the float64 pipe; pE_f, sE_f carry the column scaling (pE escale, sE escale)
+  float alpha_f, omega_f, beta_f, pE_f, sE_f;
 };
+template <typename T>
+__device__ __forceinline__ T ks_scalar(double d, float f) {
+  if constexpr (sizeof(T) == 4) return f;
+  else return d;
+}
 
 // ---- block reductions into per-block partials ------------------------------------------
 // Sum NQ doubles over the block; thread 0 writes part[q * G + blk].
@@ -131,8 +139,17 @@ __device__ __forceinline__ void block_partials_k(const TK (&v)[NQ], double *part
       if (lane == 0) red[wid][q] = (double)x;
     }
     __syncthreads();
-    if (threadIdx.x < NQ) {
-      const int nw = (blockDim.x + 31) >> 5;
+    const int nw = (blockDim.x + 31) >> 5;
+    if (NQ <= 4 && nw <= 8) {
+      // one warp, eight lanes a quantity: three dependent float64 adds
+      if (threadIdx.x < 32) {
+        const int q = threadIdx.x >> 3, w = threadIdx.x & 7;
+        double sum = q < NQ && w < nw ? red[w][q] : 0.0;
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        if (w == 0 && q < NQ) part[q * G + blk] = sum;
+      }
+    } else if (threadIdx.x < NQ) {
       double sum = 0.0;
       for (int w = 0; w < nw; ++w) sum += red[w][threadIdx.x];
       part[threadIdx.x * G + blk] = sum;
@@ -176,7 +193,8 @@ struct ApplyArgs {
   const T *tan;         // tangent channels (TanIdx)
   const double *xE_ptr; // E slot of x (device scalar)
   double e_scale;       // column scaling of the E unknown: d_E = e_scale * xE (ks == nullptr)
-  double fM[6];         // load direction (Mandel)
+  T fM[6];              // load direction (Mandel)
+  const float *xEf_ptr; // float32 solves: the scaled E slot e_scale * xE, when the scalars hold it
   cpx<T> *spec;         // spectral scratch c * rows * hx
   double *part;         // per-block partials
   // fused BiCGStab vector updates (prologue) and dots (epilogue)
