@@ -21,6 +21,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "fx.cuh"
+
 #define FFT_MAX_STAGES 14
 
 // Aligned to its full size so that one element moves as one 8-byte (float) or 16-byte
@@ -31,16 +33,49 @@ struct __align__(2 * sizeof(T)) cpx {
 };
 
 template <typename T>
-__device__ __forceinline__ cpx<T> cmul(cpx<T> a, cpx<T> b) {
+__host__ __device__ __forceinline__ cpx<T> cmul(cpx<T> a, cpx<T> b) {
   return {a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x};
 }
 template <typename T>
-__device__ __forceinline__ cpx<T> cadd(cpx<T> a, cpx<T> b) { return {a.x + b.x, a.y + b.y}; }
+__host__ __device__ __forceinline__ cpx<T> cmul_conj(cpx<T> a, cpx<T> w) {  // a * conj(w)
+  return {a.x * w.x + a.y * w.y, a.y * w.x - a.x * w.y};
+}
 template <typename T>
-__device__ __forceinline__ cpx<T> csub(cpx<T> a, cpx<T> b) { return {a.x - b.x, a.y - b.y}; }
+__host__ __device__ __forceinline__ cpx<T> cadd(cpx<T> a, cpx<T> b) { return {a.x + b.x, a.y + b.y}; }
+template <typename T>
+__host__ __device__ __forceinline__ cpx<T> csub(cpx<T> a, cpx<T> b) { return {a.x - b.x, a.y - b.y}; }
 // multiply by i * s  (s = +1 or -1)
 template <typename T>
-__device__ __forceinline__ cpx<T> cmuli(cpx<T> a, T s) { return {-s * a.y, s * a.x}; }
+__host__ __device__ __forceinline__ cpx<T> cmuli(cpx<T> a, T s) { return {-s * a.y, s * a.x}; }
+
+// Rotation of fixed-point values by a table entry (fx.cuh), and multiplication by i * s.
+__host__ __device__ __forceinline__ cpx<fx> cmul(cpx<fx> a, int4 w) {
+  cpx<fx> o;
+  fx_rotate(a.x.v, a.y.v, w, false, o.x.v, o.y.v);
+  return o;
+}
+__host__ __device__ __forceinline__ cpx<fx> cmul_conj(cpx<fx> a, int4 w) {
+  cpx<fx> o;
+  fx_rotate(a.x.v, a.y.v, w, true, o.x.v, o.y.v);
+  return o;
+}
+__host__ __device__ __forceinline__ cpx<fx> cmuli(cpx<fx> a, int s) {
+  return s > 0 ? cpx<fx>{-a.y, a.x} : cpx<fx>{a.y, -a.x};
+}
+
+// Type of a table entry and of the transform direction for values of type T.
+template <typename T>
+struct FftTypes {
+  using Tw = cpx<T>;
+  using Dir = T;
+  static constexpr bool kFixed = false;
+};
+template <>
+struct FftTypes<fx> {
+  using Tw = int4;
+  using Dir = int;
+  static constexpr bool kFixed = true;
+};
 
 // Division by a runtime constant d through a multiply-high: for x < 2^32 / d,
 // floor(x / d) = umulhi(x, ceil(2^32 / d)).  All callers divide indices below 2^20 by
@@ -68,8 +103,8 @@ __device__ __forceinline__ int smap(int e) {
 template <int NL>
 __host__ __device__ __forceinline__ constexpr int line_slots(int Np_rt) { return NL > 0 ? NL : Np_rt; }
 
-// Transform plan of one line length N.  tw points to N twiddles exp(-2 pi i k / N) of the
-// transform precision (cpx<float> or cpx<double>), rev / unrev to the digit-reversal
+// Transform plan of one line length N.  tw points to N twiddles exp(-2 pi i k / N) (cpx<float>,
+// or int4 halves of Q62 numbers for the float64 lines, fx.cuh), rev / unrev to the digit-reversal
 // permutation and its inverse (N entries each), all in global memory.
 struct FftPlan {
   int N;
@@ -86,14 +121,14 @@ struct FftPlan {
 
 // ---- R-point DFTs in registers, sign dir (-1 forward, +1 inverse) ----------------------
 template <typename T>
-__device__ __forceinline__ void dft2(cpx<T> *v) {
+__host__ __device__ __forceinline__ void dft2(cpx<T> *v) {
   cpx<T> a = v[0], b = v[1];
   v[0] = cadd(a, b);
   v[1] = csub(a, b);
 }
 
 template <typename T>
-__device__ __forceinline__ void dft3(cpx<T> *v, T dir) {
+__host__ __device__ __forceinline__ void dft3(cpx<T> *v, T dir) {
   const T s3 = (T)0.86602540378443864676;  // sin(2 pi / 3)
   cpx<T> t1 = cadd(v[1], v[2]);
   cpx<T> t2 = csub(v[1], v[2]);
@@ -105,7 +140,7 @@ __device__ __forceinline__ void dft3(cpx<T> *v, T dir) {
 }
 
 template <typename T>
-__device__ __forceinline__ void dft4(cpx<T> *v, T dir) {
+__host__ __device__ __forceinline__ void dft4(cpx<T> *v, T dir) {
   cpx<T> a = cadd(v[0], v[2]), b = csub(v[0], v[2]);
   cpx<T> c = cadd(v[1], v[3]), d = cmuli(csub(v[1], v[3]), dir);
   v[0] = cadd(a, c);
@@ -115,7 +150,7 @@ __device__ __forceinline__ void dft4(cpx<T> *v, T dir) {
 }
 
 template <typename T>
-__device__ __forceinline__ void dft8(cpx<T> *v, T dir) {
+__host__ __device__ __forceinline__ void dft8(cpx<T> *v, T dir) {
   const T h = (T)0.70710678118654752440;  // sqrt(1/2)
   cpx<T> e[4] = {v[0], v[2], v[4], v[6]};
   cpx<T> o[4] = {v[1], v[3], v[5], v[7]};
@@ -135,6 +170,59 @@ __device__ __forceinline__ void dft8(cpx<T> *v, T dir) {
   v[6] = csub(e[2], o2);
   v[3] = cadd(e[3], o3);
   v[7] = csub(e[3], o3);
+}
+
+__host__ __device__ __forceinline__ void dft3(cpx<fx> *v, int dir) {
+  cpx<fx> t1 = cadd(v[1], v[2]);
+  cpx<fx> t2 = csub(v[1], v[2]);
+  cpx<fx> m = {{v[0].x.v - (t1.x.v >> 1)}, {v[0].y.v - (t1.y.v >> 1)}};
+  cpx<fx> r = cmuli(cpx<fx>{fx_mul_sqrt3h(t2.x), fx_mul_sqrt3h(t2.y)}, dir);
+  v[0] = cadd(v[0], t1);
+  v[1] = cadd(m, r);
+  v[2] = csub(m, r);
+}
+
+__host__ __device__ __forceinline__ void dft4(cpx<fx> *v, int dir) {
+  cpx<fx> a = cadd(v[0], v[2]), b = csub(v[0], v[2]);
+  cpx<fx> c = cadd(v[1], v[3]), d = cmuli(csub(v[1], v[3]), dir);
+  v[0] = cadd(a, c);
+  v[2] = csub(a, c);
+  v[1] = cadd(b, d);
+  v[3] = csub(b, d);
+}
+
+__host__ __device__ __forceinline__ void dft8(cpx<fx> *v, int dir) {
+  cpx<fx> e[4] = {v[0], v[2], v[4], v[6]};
+  cpx<fx> o[4] = {v[1], v[3], v[5], v[7]};
+  dft4(e, dir);
+  dft4(o, dir);
+  // W8 and W8^3: 45 degree rotations, one real product a component
+  const cpx<fx> i1 = cmuli(o[1], dir), i3 = cmuli(o[3], dir);
+  const cpx<fx> a1 = cadd(o[1], i1), a3 = csub(i3, o[3]);
+  const cpx<fx> o1 = {fx_mul_rsqrt2(a1.x), fx_mul_rsqrt2(a1.y)};
+  const cpx<fx> o2 = cmuli(o[2], dir);
+  const cpx<fx> o3 = {fx_mul_rsqrt2(a3.x), fx_mul_rsqrt2(a3.y)};
+  v[0] = cadd(e[0], o[0]);
+  v[4] = csub(e[0], o[0]);
+  v[1] = cadd(e[1], o1);
+  v[5] = csub(e[1], o1);
+  v[2] = cadd(e[2], o2);
+  v[6] = csub(e[2], o2);
+  v[3] = cadd(e[3], o3);
+  v[7] = csub(e[3], o3);
+}
+
+// the shift after stage s of a fixed-point line (nothing in floating point)
+template <typename T, int R>
+__device__ __forceinline__ void stage_shift(cpx<T> (&v)[R], const unsigned long long *meta, int line, int s) {
+  if constexpr (FftTypes<T>::kFixed) {
+    const int sh = fx_shift(meta[line], s);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      v[r].x.v = fx_round_shift(v[r].x.v, sh);
+      v[r].y.v = fx_round_shift(v[r].y.v, sh);
+    }
+  }
 }
 
 // Addressing of line l, element e in shared memory (padded element index):
@@ -160,12 +248,13 @@ __device__ __forceinline__ int line_base(const LineLayout &ly, int l) {
 // dir = -1 forward, +1 inverse.  Caller syncs between stages.
 template <typename T, bool DIT, int R>
 __device__ __forceinline__ void fft_stage_r(cpx<T> *sm, const LineLayout &ly, const FftPlan &pl, int s,
-                                            T dir) {
+                                            typename FftTypes<T>::Dir dir, const unsigned long long *meta) {
+  using Tw = typename FftTypes<T>::Tw;
   const int N = pl.N, Ns = pl.Ns[s];
   const int nb = N / R;
   const int tot = ly.L * nb;
   const int twstep = N / (Ns * R);
-  const cpx<T> *tw = (const cpx<T> *)pl.tw;
+  const Tw *tw = (const Tw *)pl.tw;
   for (int b = threadIdx.x; b < tot; b += blockDim.x) {
     int l, q;
     if (ly.line_fastest) {
@@ -185,9 +274,9 @@ __device__ __forceinline__ void fft_stage_r(cpx<T> *sm, const LineLayout &ly, co
     if (DIT && j != 0) {
 #pragma unroll
       for (int r = 1; r < R; ++r) {
-        cpx<T> w = tw[r * j * twstep];  // index < R * Ns * N / (Ns * R) = N
-        w.y *= -dir;  // table holds exp(-2 pi i e/N); dir = +1 needs the conjugate
-        v[r] = cmul(v[r], w);
+        const Tw w = tw[r * j * twstep];  // index < R * Ns * N / (Ns * R) = N
+        // the table holds exp(-2 pi i e/N); the inverse transform needs the conjugate
+        v[r] = cmul_conj(v[r], w);
       }
     }
     if (R == 8) dft8(v, dir);
@@ -197,40 +286,41 @@ __device__ __forceinline__ void fft_stage_r(cpx<T> *sm, const LineLayout &ly, co
     if (!DIT && j != 0) {
 #pragma unroll
       for (int r = 1; r < R; ++r) {
-        cpx<T> w = tw[r * j * twstep];
-        w.y *= -dir;
+        const Tw w = tw[r * j * twstep];
         v[r] = cmul(v[r], w);
       }
     }
+    stage_shift<T, R>(v, meta, l, s);
 #pragma unroll
     for (int r = 0; r < R; ++r) sm[lb + pad8(e0 + r * Ns) * ly.es] = v[r];
   }
 }
 
 template <typename T, bool DIT>
-__device__ __forceinline__ void fft_stage(cpx<T> *sm, const LineLayout &ly, const FftPlan &pl, int s, T dir) {
+__device__ __forceinline__ void fft_stage(cpx<T> *sm, const LineLayout &ly, const FftPlan &pl, int s,
+                                          typename FftTypes<T>::Dir dir, const unsigned long long *meta) {
   switch (pl.R[s]) {
-    case 8: fft_stage_r<T, DIT, 8>(sm, ly, pl, s, dir); break;
-    case 4: fft_stage_r<T, DIT, 4>(sm, ly, pl, s, dir); break;
-    case 3: fft_stage_r<T, DIT, 3>(sm, ly, pl, s, dir); break;
-    case 2: fft_stage_r<T, DIT, 2>(sm, ly, pl, s, dir); break;
+    case 8: fft_stage_r<T, DIT, 8>(sm, ly, pl, s, dir, meta); break;
+    case 4: fft_stage_r<T, DIT, 4>(sm, ly, pl, s, dir, meta); break;
+    case 3: fft_stage_r<T, DIT, 3>(sm, ly, pl, s, dir, meta); break;
+    case 2: fft_stage_r<T, DIT, 2>(sm, ly, pl, s, dir, meta); break;
     default: break;  // N = 1
   }
 }
 
 // Full DIF transform of all lines (natural in, digit-reversed out).
 template <typename T>
-__device__ void fft_dif(cpx<T> *sm, const LineLayout &ly, const FftPlan &pl, T dir) {
+__device__ void fft_dif(cpx<T> *sm, const LineLayout &ly, const FftPlan &pl, const unsigned long long *meta = nullptr) {
   for (int s = pl.S - 1; s >= 0; --s) {
-    fft_stage<T, false>(sm, ly, pl, s, dir);
+    fft_stage<T, false>(sm, ly, pl, s, -1, meta);
     __syncthreads();
   }
 }
 // Full DIT transform (digit-reversed in, natural out).
 template <typename T>
-__device__ void fft_dit(cpx<T> *sm, const LineLayout &ly, const FftPlan &pl, T dir) {
+__device__ void fft_dit(cpx<T> *sm, const LineLayout &ly, const FftPlan &pl, const unsigned long long *meta = nullptr) {
   for (int s = 0; s < pl.S; ++s) {
-    fft_stage<T, true>(sm, ly, pl, s, dir);
+    fft_stage<T, true>(sm, ly, pl, s, 1, meta);
     __syncthreads();
   }
 }
@@ -262,16 +352,12 @@ __host__ __device__ constexpr StagePlan stage_plan(int N) {
   return p;
 }
 
-template <typename T>
-__device__ __forceinline__ cpx<T> cmul_conj(cpx<T> a, cpx<T> w) {  // a * conj(w)
-  return {a.x * w.x + a.y * w.y, a.y * w.x - a.x * w.y};
-}
-
 // Twiddles w[r] = tw[r * jt], r = 1..R-1, of one butterfly.  For float32 radix 8 only
 // w1, w2, w4 are loaded and w3, w5, w6, w7 formed as products of two of them (at most one
 // extra rounding), which halves the table traffic through L1.
 template <typename T, int R>
-__device__ __forceinline__ void load_twiddles(const cpx<T> *__restrict__ tw, int jt, cpx<T> (&w)[R]) {
+__device__ __forceinline__ void load_twiddles(const typename FftTypes<T>::Tw *__restrict__ tw, int jt,
+                                              typename FftTypes<T>::Tw (&w)[R]) {
   if constexpr (R == 8 && sizeof(T) == 4) {
     w[1] = tw[jt];
     w[2] = tw[2 * jt];
@@ -291,13 +377,15 @@ __device__ __forceinline__ void load_twiddles(const cpx<T> *__restrict__ tw, int
 // LW >= 0 fixes lw at compile time (x passes: 0); LW < 0 takes the runtime lw.
 // INV: inverse (DIT, twiddle before the DFT, conjugate twiddles); else forward (DIF).
 template <typename T, bool INV, int R, int NS, int N, int LW>
-__device__ __forceinline__ void ct_stage(cpx<T> *sm, int Lc, int lw_rt, const cpx<T> *__restrict__ tw) {
+__device__ __forceinline__ void ct_stage(cpx<T> *sm, int Lc, int lw_rt,
+                                         const typename FftTypes<T>::Tw *__restrict__ tw,
+                                         const unsigned long long *meta = nullptr, int s = 0) {
   constexpr int NB = N / R;
   constexpr int TWS = N / (NS * R);
   constexpr int Np = N;  // swizzled lines (smap), no padding
   const int lw = LW >= 0 ? LW : lw_rt;
   const int tot = (Lc * NB) << lw;
-  const T dir = INV ? (T)1 : (T)-1;
+  const typename FftTypes<T>::Dir dir = INV ? 1 : -1;
   for (int b = threadIdx.x; b < tot; b += blockDim.x) {
     const int w = b & ((1 << lw) - 1);
     const int rest = b >> lw;
@@ -314,7 +402,7 @@ __device__ __forceinline__ void ct_stage(cpx<T> *sm, int Lc, int lw_rt, const cp
     cpx<T> v[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) v[r] = base[off[r]];
-    cpx<T> wt[R];
+    typename FftTypes<T>::Tw wt[R];
     if constexpr (NS > 1) load_twiddles<T, R>(tw, j * TWS, wt);
     if constexpr (INV && NS > 1) {
 #pragma unroll
@@ -328,28 +416,31 @@ __device__ __forceinline__ void ct_stage(cpx<T> *sm, int Lc, int lw_rt, const cp
 #pragma unroll
       for (int r = 1; r < R; ++r) v[r] = cmul(v[r], wt[r]);
     }
+    stage_shift<T, R>(v, meta, (lc << lw) + w, s);
 #pragma unroll
     for (int r = 0; r < R; ++r) base[off[r]] = v[r];
   }
 }
 
 template <typename T, int N, int LW, int s>
-__device__ __forceinline__ void ct_dif_from(cpx<T> *sm, int Lc, int lw, const cpx<T> *tw) {
+__device__ __forceinline__ void ct_dif_from(cpx<T> *sm, int Lc, int lw, const typename FftTypes<T>::Tw *tw,
+                                            const unsigned long long *meta = nullptr) {
   if constexpr (s >= 0) {
     constexpr StagePlan P = stage_plan(N);
-    ct_stage<T, false, P.R[s], P.Ns[s], N, LW>(sm, Lc, lw, tw);
+    ct_stage<T, false, P.R[s], P.Ns[s], N, LW>(sm, Lc, lw, tw, meta, s);
     __syncthreads();
-    ct_dif_from<T, N, LW, s - 1>(sm, Lc, lw, tw);
+    ct_dif_from<T, N, LW, s - 1>(sm, Lc, lw, tw, meta);
   }
 }
 
 template <typename T, int N, int LW, int s>
-__device__ __forceinline__ void ct_dit_from(cpx<T> *sm, int Lc, int lw, const cpx<T> *tw) {
+__device__ __forceinline__ void ct_dit_from(cpx<T> *sm, int Lc, int lw, const typename FftTypes<T>::Tw *tw,
+                                            const unsigned long long *meta = nullptr) {
   constexpr StagePlan P = stage_plan(N);
   if constexpr (s < P.S) {
-    ct_stage<T, true, P.R[s], P.Ns[s], N, LW>(sm, Lc, lw, tw);
+    ct_stage<T, true, P.R[s], P.Ns[s], N, LW>(sm, Lc, lw, tw, meta, s);
     __syncthreads();
-    ct_dit_from<T, N, LW, s + 1>(sm, Lc, lw, tw);
+    ct_dit_from<T, N, LW, s + 1>(sm, Lc, lw, tw, meta);
   }
 }
 
@@ -357,13 +448,15 @@ __device__ __forceinline__ void ct_dit_from(cpx<T> *sm, int Lc, int lw, const cp
 // out) of Lc * 2^lw lines of compile-time length N; same operations and order as
 // fft_dif / fft_dit with the host plan of N.
 template <typename T, int N, int LW>
-__device__ __forceinline__ void fft_dif_ct(cpx<T> *sm, int Lc, int lw, const cpx<T> *tw) {
+__device__ __forceinline__ void fft_dif_ct(cpx<T> *sm, int Lc, int lw, const typename FftTypes<T>::Tw *tw,
+                                            const unsigned long long *meta = nullptr) {
   constexpr StagePlan P = stage_plan(N);
-  ct_dif_from<T, N, LW, P.S - 1>(sm, Lc, lw, tw);
+  ct_dif_from<T, N, LW, P.S - 1>(sm, Lc, lw, tw, meta);
 }
 template <typename T, int N, int LW>
-__device__ __forceinline__ void fft_dit_ct(cpx<T> *sm, int Lc, int lw, const cpx<T> *tw) {
-  ct_dit_from<T, N, LW, 0>(sm, Lc, lw, tw);
+__device__ __forceinline__ void fft_dit_ct(cpx<T> *sm, int Lc, int lw, const typename FftTypes<T>::Tw *tw,
+                                            const unsigned long long *meta = nullptr) {
+  ct_dit_from<T, N, LW, 0>(sm, Lc, lw, tw, meta);
 }
 
 // Digit reversal of the compile-time plan of N: position -> sample / frequency index (rev)

@@ -19,6 +19,8 @@
 //   3D: x-forward -> y-forward -> z fused -> y-inverse -> x-inverse   5 kernels
 // Two real rows are transformed together as one complex row (z = a + i b) and separated
 // by Hermitian symmetry, so every FFT in the x passes is a full-length complex FFT.
+#include <type_traits>
+
 #include "rve_kern.cuh"
 #include "krylov_fin.cuh"
 
@@ -93,6 +95,141 @@ __device__ __forceinline__ void willot_n(const AxisTab<T> &tb, const int *k, T *
   }
 }
 
+// ---- float64 lines in block fixed point (fx.cuh) ----------------------------------------
+// Lines lie in shared memory as ((lc Np + smap(e)) << lw) + w (lc < Lc groups of 2^lw adjacent
+// lines, Np slots a line); the state of line (lc, w) is meta[(lc << lw) + w], after the lines.
+// The float64 lines are replaced in place by integers: one sweep finds each line's largest
+// exponent, a second aligns the values to it and sums their magnitudes.  nw / Lc warps share a
+// group where there are fewer groups than warps, else a warp takes whole groups.  Starts
+// and ends with a barrier.
+__device__ __forceinline__ unsigned long long *fx_meta(cpx<double> *sm, int Lc, int lw, int Np) {
+  return reinterpret_cast<unsigned long long *>(sm + ((Lc * Np) << lw));
+}
+
+template <int NL>
+__device__ __forceinline__ void fx_load_lines(cpx<double> *sm, int Lc, int lw, int Np, const FftPlan &pl, bool inverse) {
+  __shared__ unsigned long long acc[32][16];
+  const int N = NL > 0 ? NL : pl.N;
+  unsigned long long *meta = fx_meta(sm, Lc, lw, Np);
+  const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int W = 1 << lw, w = lane & (W - 1);
+  const int spl = Lc < nw ? nw / Lc : 1;  // warps per group
+  const int step = (32 >> lw) * spl;
+  const unsigned long long *raw = reinterpret_cast<const unsigned long long *>(sm);
+  longlong2 *out = reinterpret_cast<longlong2 *>(sm);
+  __syncthreads();
+  const int part = wi % spl;
+  for (int lc = wi / spl;; lc += nw / spl) {
+    const bool on = lc < Lc;
+    if (!on && spl == 1) break;
+    const int e0 = (lane >> lw) + part * (32 >> lw);
+    const int base = lc * Np;
+    unsigned mx = 0;
+    if (on) {
+#pragma unroll 4
+      for (int e = e0; e < N; e += step) {
+        const int o = ((base + smap<NL>(e)) << lw) + w;
+        const ulonglong2 z = reinterpret_cast<const ulonglong2 *>(raw)[o];
+        mx = max(mx, max((unsigned)(z.x >> 32) & 0x7FFFFFFFu, (unsigned)(z.y >> 32) & 0x7FFFFFFFu));
+      }
+      for (int o = W; o < 32; o <<= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    }
+    if (spl > 1) {
+      if (on && lane < W) acc[wi][w] = mx;
+      __syncthreads();
+      if (on)
+        for (int k = 0; k < spl; ++k) mx = max(mx, (unsigned)acc[wi - part + k][w]);
+    }
+    const int E = max((int)(mx >> 20), 1);
+    unsigned long long sum = 0;
+    if (on) {
+#pragma unroll 4
+      for (int e = e0; e < N; e += step) {
+        const int o = ((base + smap<NL>(e)) << lw) + w;
+        const ulonglong2 z = reinterpret_cast<const ulonglong2 *>(raw)[o];
+        const long long a = fx_from_bits(z.x, E), b = fx_from_bits(z.y, E);
+        out[o] = make_longlong2(a, b);
+        sum += (unsigned long long)((a < 0 ? -a : a) + (b < 0 ? -b : b)) >> 16;
+      }
+      for (int o = W; o < 32; o <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    }
+    if (spl > 1) {
+      __syncthreads();  // the maxima have been read
+      if (on && lane < W) acc[wi][w] = sum;
+      __syncthreads();
+      if (on && part == 0)
+        for (int k = 1; k < spl; ++k) sum += acc[wi + k][w];
+    }
+    if (on && part == 0 && lane < W) {
+      const int lsum = 80 - __clzll((long long)(sum + N));
+      unsigned long long state;
+      if constexpr (NL > 0) {
+        constexpr StagePlan P = stage_plan(NL);
+        state = inverse ? fx_schedule(P.R, P.S, true, lsum, E) : fx_schedule(P.R, P.S, false, lsum, E);
+      } else {
+        state = fx_schedule(pl.R, pl.S, inverse, lsum, E);
+      }
+      meta[(lc << lw) + w] = state;
+    }
+    if (spl > 1) break;  // every group has its warps
+  }
+  __syncthreads();
+}
+
+// one value of a transformed line in type T: of integers scaled by the line's exponent
+template <typename T>
+__device__ __forceinline__ cpx<T> line_value(cpx<T> z, const unsigned long long *meta, int line) {
+  if constexpr (sizeof(T) == 8) {
+    const int e = fx_exp(meta[line]);
+    if (e == kFxNonFinite) {  // a NaN or an infinity anywhere in a line reaches all of its values
+      const T nan = __longlong_as_double(0x7FF8000000000000ll);
+      return {nan, nan};
+    }
+    return {__longlong_as_double((long long)fx_to_bits(__double_as_longlong(z.x), e)),
+            __longlong_as_double((long long)fx_to_bits(__double_as_longlong(z.y), e))};
+  } else {
+    return z;
+  }
+}
+
+// Transforms of Lc 2^lw lines in shared memory; float64 lines enter as float64 and leave as
+// fixed point (read through line_value).
+template <typename T, int NL, bool INV, int LW>
+__device__ __forceinline__ void fft_lines(cpx<T> *sm, int Lc, int lw, const FftPlan &pl) {
+  constexpr bool fixed = sizeof(T) == 8;
+  const int Np = line_slots<NL>(pl.Np);
+  const unsigned long long *meta = nullptr;
+  if constexpr (fixed) {
+    fx_load_lines<NL>(sm, Lc, lw, Np, pl, INV);
+    meta = fx_meta(sm, Lc, lw, Np);
+  } else {
+    __syncthreads();
+  }
+  using V = std::conditional_t<fixed, fx, T>;
+  cpx<V> *lines = reinterpret_cast<cpx<V> *>(sm);
+  if constexpr (NL > 0) {
+    const auto *tw = (const typename FftTypes<V>::Tw *)pl.tw;
+    if constexpr (INV) fft_dit_ct<V, NL, LW>(lines, Lc, lw, tw, meta);
+    else fft_dif_ct<V, NL, LW>(lines, Lc, lw, tw, meta);
+  } else {
+    // lw > 0: consecutive threads take consecutive lines (contiguous addresses); lw = 0: the
+    // lines are Np apart, a multiple of the bank count for power-of-two N, so consecutive
+    // threads take consecutive butterflies of one line instead
+    const int W = 1 << lw;
+    LineLayout ly;
+    ly.L = Lc << lw;
+    ly.dL = make_fdiv(Lc << lw);
+    ly.lw = W;
+    ly.dlw = make_fdiv(W);
+    ly.lsA = Np << lw;
+    ly.lsB = 1;
+    ly.es = W;
+    ly.line_fastest = lw > 0;
+    if constexpr (INV) fft_dit<V>(lines, ly, pl, meta);
+    else fft_dif<V>(lines, ly, pl, meta);
+  }
+}
+
 // ---- x-forward tail: DIF over the packed row pairs, then Hermitian unpack + store -------
 // tr = 0: half spectra stored row-major [ch][row][kx] (coalesced along kx);
 // tr = 1: stored transposed [ch][kx][row] for the fused 2D column pass (k_col_fused2d).
@@ -103,22 +240,12 @@ template <typename T, int NL>
 __device__ __forceinline__ void xfwd_tail(cpx<T> *sm, int c, int P, int row0, const Geo &g, const FftPlan &pl,
                           cpx<T> *spec, int tr = 0) {
   const int nx = NL > 0 ? NL : g.nx, hx = nx / 2 + 1, Np = line_slots<NL>(pl.Np);
-  __syncthreads();
-  if constexpr (NL > 0) {
-    fft_dif_ct<T, NL, 0>(sm, c * P, 0, (const cpx<T> *)pl.tw);
-  } else {
-    LineLayout ly;
-    ly.L = c * P;
-    ly.lw = 1;
-    ly.lsA = Np;
-    ly.lsB = 0;
-    ly.es = 1;
-    ly.line_fastest = false;
-    fft_dif<T>(sm, ly, pl, (T)-1);
-  }
+  fft_lines<T, NL, false, 0>(sm, c * P, 0, pl);
+  [[maybe_unused]] const unsigned long long *meta = nullptr;
+  if constexpr (sizeof(T) == 8) meta = fx_meta(sm, c * P, 0, Np);
   const int cs = g.rows * hx;
   const FDiv dhx = make_fdiv(hx), dP = make_fdiv(P);
-  if (tr) {
+  if (sizeof(T) == 4 && tr) {
     const int totp = c * P * nx;
     const FDiv dnx = make_fdiv(nx);
     for (int i = threadIdx.x; i < totp; i += blockDim.x) {
@@ -159,8 +286,17 @@ __device__ __forceinline__ void xfwd_tail(cpx<T> *sm, int c, int P, int row0, co
     const int ch = (int)fdiv(l, dP), pr = l - ch * P;
     const cpx<T> zk = sm[l * Np + smap<NL>(pl.unrev[k])];
     const cpx<T> zn = sm[l * Np + smap<NL>(pl.unrev[k == 0 ? 0 : nx - k])];
-    const cpx<T> A = {(zk.x + zn.x) * (T)0.5, (zk.y - zn.y) * (T)0.5};
-    const cpx<T> B = {(zk.y + zn.y) * (T)0.5, (zn.x - zk.x) * (T)0.5};
+    cpx<T> A, B;
+    if constexpr (sizeof(T) == 8) {
+      // halves of sums of integers
+      const long long kx = __double_as_longlong(zk.x) >> 1, ky = __double_as_longlong(zk.y) >> 1;
+      const long long mx = __double_as_longlong(zn.x) >> 1, my = __double_as_longlong(zn.y) >> 1;
+      A = line_value<T>({__longlong_as_double(kx + mx), __longlong_as_double(ky - my)}, meta, l);
+      B = line_value<T>({__longlong_as_double(ky + my), __longlong_as_double(mx - kx)}, meta, l);
+    } else {
+      A = {(zk.x + zn.x) * (T)0.5, (zk.y - zn.y) * (T)0.5};
+      B = {(zk.y + zn.y) * (T)0.5, (zn.x - zk.x) * (T)0.5};
+    }
     const int r0 = row0 + 2 * pr, r1 = r0 + 1;
     if (r0 < g.rows) spec[ch * cs + r0 * hx + k] = A;
     if (r1 < g.rows) spec[ch * cs + r1 * hx + k] = B;
@@ -175,7 +311,7 @@ __device__ __forceinline__ void xinv_head(cpx<T> *sm, int c, int P, int row0, co
   const int cs = g.rows * hx;
   const int tot = c * P * hx;
   const FDiv dhx = make_fdiv(hx), dP = make_fdiv(P);
-  if (tr) {
+  if (sizeof(T) == 4 && tr) {
     // Z_k = A + iB for k <= nx/2 and Z_{nx-k} = conj(A) + i conj(B), with (A, B) the half-
     // spectrum entries of the row pair at k.  Threads walk the positions p of each line
     // (k = rev(p)); a position with k <= nx/2 loads its entry once and writes both p and the
@@ -254,19 +390,7 @@ __device__ __forceinline__ void xinv_head(cpx<T> *sm, int c, int P, int row0, co
     sm[l * Np + smap<NL>(pl.unrev[k])] = {A.x - B.y, A.y + B.x};
     if (k > 0 && 2 * k < nx) sm[l * Np + smap<NL>(pl.unrev[nx - k])] = {A.x + B.y, B.x - A.y};
   }
-  __syncthreads();
-  if constexpr (NL > 0) {
-    fft_dit_ct<T, NL, 0>(sm, c * P, 0, (const cpx<T> *)pl.tw);
-  } else {
-    LineLayout ly;
-    ly.L = c * P;
-    ly.lw = 1;
-    ly.lsA = Np;
-    ly.lsB = 0;
-    ly.es = 1;
-    ly.line_fastest = false;
-    fft_dit<T>(sm, ly, pl, (T)1);
-  }
+  fft_lines<T, NL, true, 0>(sm, c * P, 0, pl);
 }
 
 }  // namespace
@@ -526,6 +650,8 @@ __global__ void __launch_bounds__(256) k_xinv_apply(const __grid_constant__ Appl
   const int row0 = blockIdx.x * 2 * P;
   const FDiv dnx = make_fdiv(nx);
   xinv_head<T, NL>(sm, c, P, row0, g, pl, a.spec, a.tr);
+  [[maybe_unused]] const unsigned long long *meta = nullptr;
+  if constexpr (sizeof(T) == 8) meta = fx_meta(sm, c * P, 0, Np);
   T d[5] = {0, 0, 0, 0, 0};  // per-thread and warp sums in T, block and grid sums in float64
   const int tot = P * nx;
   for (int i = threadIdx.x; i < tot; i += blockDim.x) {
@@ -540,7 +666,7 @@ __global__ void __launch_bounds__(256) k_xinv_apply(const __grid_constant__ Appl
     T y0[M + 1], y1[M + 1];
 #pragma unroll
     for (int k = 0; k <= M; ++k) {
-      const cpx<T> z = sm[(k * P + l0) * Np + px];
+      const cpx<T> z = line_value<T>(sm[(k * P + l0) * Np + px], meta, k * P + l0);
       y0[k] = z.x;
       y1[k] = z.y;
     }
@@ -624,24 +750,10 @@ __global__ void __launch_bounds__(256) k_col(const __grid_constant__ ColGroup<T>
     for (int u = 0; u < KU; ++u)
       if (slot[u] >= 0) sm[slot[u]] = val[u];
   }
-  __syncthreads();
-  LineLayout ly;
-  ly.L = c * W;
-  ly.dL = make_fdiv(c * W);
-  ly.lw = W;
-  ly.dlw = make_fdiv(W);
-  ly.lsA = Np * W;
-  ly.lsB = 1;
-  ly.es = W;
-  // W > 1: consecutive threads take consecutive columns (contiguous addresses); W = 1: the
-  // lines (channels) are Np apart, a multiple of the bank count for power-of-two N, so
-  // consecutive threads take consecutive butterflies of one line instead
-  ly.line_fastest = W > 1;
-  const cpx<T> *tw = (const cpx<T> *)a.plan.tw;
-  if (MODE == 0 || MODE == 1) {
-    if constexpr (NL > 0) fft_dif_ct<T, NL, -1>(sm, c, lw, tw);
-    else fft_dif<T>(sm, ly, a.plan, (T)-1);
-  }
+  // (fft_lines starts with a barrier)
+  [[maybe_unused]] const unsigned long long *meta = nullptr;
+  if constexpr (sizeof(T) == 8) meta = fx_meta(sm, c, lw, Np);
+  if (MODE == 0 || MODE == 1) fft_lines<T, NL, false, -1>(sm, c, lw, a.plan);
   if (MODE == 1) {
     constexpr int D = (M == 3) ? 2 : 3;
     const int ky_other = (D == 3) ? a.yplan.rev[other] : 0;
@@ -663,7 +775,7 @@ __global__ void __launch_bounds__(256) k_col(const __grid_constant__ ColGroup<T>
       T re[M], im[M];
 #pragma unroll
       for (int ch = 0; ch < M; ++ch) {
-        const cpx<T> z = sm[((ch * Np + pp) << lw) + w];
+        const cpx<T> z = line_value<T>(sm[((ch * Np + pp) << lw) + w], meta, (ch << lw) + w);
         re[ch] = z.x;
         im[ch] = z.y;
       }
@@ -671,22 +783,20 @@ __global__ void __launch_bounds__(256) k_col(const __grid_constant__ ColGroup<T>
       project_mandel<T, M>(im, nv, a.inv_n);
 #pragma unroll
       for (int ch = 0; ch < M; ++ch) sm[((ch * Np + pp) << lw) + w] = {re[ch], im[ch]};
-      cpx<T> zp = sm[((M * Np + pp) << lw) + w];
+      const cpx<T> zp = line_value<T>(sm[((M * Np + pp) << lw) + w], meta, (M << lw) + w);
       const T sc = xi2 * a.inv_n;
       sm[((M * Np + pp) << lw) + w] = {zp.x * sc, zp.y * sc};
     }
-    __syncthreads();
   }
-  if (MODE == 1 || MODE == 2) {
-    if constexpr (NL > 0) fft_dit_ct<T, NL, -1>(sm, c, lw, tw);
-    else fft_dit<T>(sm, ly, a.plan, (T)1);
-  }
+  if (MODE == 1 || MODE == 2) fft_lines<T, NL, true, -1>(sm, c, lw, a.plan);
   for (int i = threadIdx.x; i < tot; i += blockDim.x) {
     const int iw = i >> lw;
     const int w = i & (W - 1);
     const int ch = NL > 0 ? iw / NL : (int)fdiv(iw, dN);
     const int e = iw - ch * N;
-    if (kx0 + w < g.hx) spec[ch * cs + base_o + e * es_g + kx0 + w] = sm[((ch * Np + smap<NL>(e)) << lw) + w];
+    if (kx0 + w < g.hx)
+      spec[ch * cs + base_o + e * es_g + kx0 + w] =
+          line_value<T>(sm[((ch * Np + smap<NL>(e)) << lw) + w], meta, (ch << lw) + w);
   }
 }
 

@@ -48,6 +48,7 @@ __global__ void __launch_bounds__(256) k_xinv_resid(ResidArgs a, FftPlan pl, int
   const int row0 = blockIdx.x * 2 * P;
   const FDiv dnx = make_fdiv(nx);
   xinv_head<double, 0>(sm, c, P, row0, g, pl, a.spec);
+  const unsigned long long *meta = fx_meta(sm, c * P, 0, Np);
   double acc[5] = {0, 0, 0, 0, 0};
   const int tot = 2 * P * nx;
   const double ell = a.ell;
@@ -62,7 +63,7 @@ __global__ void __launch_bounds__(256) k_xinv_resid(ResidArgs a, FftPlan pl, int
     double val[M + 1];
 #pragma unroll
     for (int k = 0; k <= M; ++k) {
-      const cpx<double> z = sm[(k * P + l0) * Np + px];
+      const cpx<double> z = line_value<double>(sm[(k * P + l0) * Np + px], meta, k * P + l0);
       val[k] = odd ? z.y : z.x;
     }
     const uint8_t mb = a.mat[v];
@@ -114,6 +115,7 @@ __global__ void __launch_bounds__(256) k_xinv_proj(ResidArgs a, FftPlan pl, int 
   const int row0 = blockIdx.x * 2 * P;
   const FDiv dnx = make_fdiv(nx);
   xinv_head<double, 0>(sm, c, P, row0, g, pl, a.spec);
+  const unsigned long long *meta = fx_meta(sm, c * P, 0, Np);
   const int tot = 2 * P * nx;
   for (int i = threadIdx.x; i < tot; i += blockDim.x) {
     const int rr = (int)fdiv(i, dnx), x = i - rr * nx;
@@ -124,7 +126,7 @@ __global__ void __launch_bounds__(256) k_xinv_proj(ResidArgs a, FftPlan pl, int 
     const int px = pad8(x);
 #pragma unroll
     for (int k = 0; k < M; ++k) {
-      const cpx<double> z = sm[(k * P + (rr >> 1)) * Np + px];
+      const cpx<double> z = line_value<double>(sm[(k * P + (rr >> 1)) * Np + px], meta, k * P + (rr >> 1));
       eps[k * n + v] = odd ? z.y : z.x;
     }
   }

@@ -243,7 +243,7 @@ static bool graphs_enabled() {
 
 // ---- the handle ------------------------------------------------------------------------
 struct DevPlan {
-  FftPlan pf, pd;  // float / double twiddles
+  FftPlan pf, pd;  // float32 twiddles / fixed-point ones (float64 lines)
 };
 
 struct Partials {
@@ -431,12 +431,21 @@ static int make_plan(rve *h, int N, DevPlan &dp, void **twd, void **twf, short *
     set_err(h, "grid extent %d is not of the form 2^a 3^b <= 4096", N);
     return RVE_E_ARG;
   }
-  std::vector<double2> td(N);
+  std::vector<int4> td(N);
   std::vector<float2> tf(N);
+  // halves of a Q62 number (fx.cuh): hi 2^32 + lo, lo > -2^31
+  auto halves = [](long double x, int &hi, int &lo) {
+    long long q = llrintl(x * 0x1p62L);
+    if ((int)q == INT32_MIN) q += 1;
+    hi = (int)((q + 0x80000000ll) >> 32);
+    lo = (int)q;
+  };
   for (int k = 0; k < N; ++k) {
     const double a = 2.0 * M_PI * (double)k / (double)N;
-    td[k] = make_double2(cos(a), -sin(a));
-    tf[k] = make_float2((float)td[k].x, (float)td[k].y);
+    tf[k] = make_float2((float)cos(a), (float)-sin(a));
+    const long double al = 2.0L * acosl(-1.0L) * (long double)k / (long double)N;
+    halves(cosl(al), td[k].x, td[k].y);
+    halves(-sinl(al), td[k].z, td[k].w);
   }
   std::vector<short> pr(2 * N);
   for (int p = 0; p < N; ++p) {
@@ -444,10 +453,10 @@ static int make_plan(rve *h, int N, DevPlan &dp, void **twd, void **twf, short *
     pr[p] = (short)r;        // rev: position -> index
     pr[N + r] = (short)p;    // unrev: index -> position
   }
-  CK(cudaMallocAsync(twd, sizeof(double2) * N, 0));
+  CK(cudaMallocAsync(twd, sizeof(int4) * N, 0));
   CK(cudaMallocAsync(twf, sizeof(float2) * N, 0));
   CK(cudaMallocAsync((void **)perm, sizeof(short) * 2 * N, 0));
-  CK(cudaMemcpy(*twd, td.data(), sizeof(double2) * N, cudaMemcpyHostToDevice));
+  CK(cudaMemcpy(*twd, td.data(), sizeof(int4) * N, cudaMemcpyHostToDevice));
   CK(cudaMemcpy(*twf, tf.data(), sizeof(float2) * N, cudaMemcpyHostToDevice));
   CK(cudaMemcpy(*perm, pr.data(), sizeof(short) * 2 * N, cudaMemcpyHostToDevice));
   pl.rev = *perm;
@@ -589,7 +598,9 @@ static void pass_geometry(const Geo &g, int es, int Preq, int Wreq, int &P, int 
   if (2 * P > g.rows + 1) P = (g.rows + 1) / 2;
   if (P < 1) P = 1;
   Gx = (g.rows + 2 * P - 1) / (2 * P);
-  smx = (size_t)g.c * P * npx * 2 * es;
+  // float64 lines carry 8 bytes of state each (fx_meta)
+  const size_t st = es == 8 ? 8 : 0;
+  smx = (size_t)g.c * P * (npx * 2 * es + st);
   auto colW = [&](int N) {
     size_t per = (size_t)g.c * padded(N) * 2 * es;  // one column, all channels, complex
     size_t w = Wreq > 0 ? (size_t)Wreq : budget / per;
@@ -602,8 +613,8 @@ static void pass_geometry(const Geo &g, int es, int Preq, int Wreq, int &P, int 
   };
   Wy = colW(g.ny);
   Wz = g.nz > 1 ? colW(g.nz) : 1;
-  smy = (size_t)g.c * padded(g.ny) * Wy * 2 * es;
-  smz = (size_t)g.c * padded(g.nz) * Wz * 2 * es;
+  smy = (size_t)g.c * Wy * (padded(g.ny) * 2 * es + st);
+  smz = (size_t)g.c * Wz * (padded(g.nz) * 2 * es + st);
 }
 
 // Opt every FFT-pass kernel in to the largest dynamic shared memory the device allows
