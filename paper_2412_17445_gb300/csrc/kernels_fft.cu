@@ -69,35 +69,34 @@ __global__ void __launch_bounds__(256) k_xinv_resid(ResidArgs a, FftPlan pl, int
     const uint8_t mb = a.mat[v];
     const bool notch = (mb & RVE_NOTCH_BIT) != 0;
     const int ph = mb & 0x7f;
-    const double Gc = a.ph.Gc[ph];
-    const double phi = a.phi[v], H = a.H[v], Lp = val[M];
-    const double aa = Gc / ell + 2.0 * H;
-    const double F2 = notch ? (phi - 1.0) : (aa * phi + Gc * ell * Lp - 2.0 * H);
-    const double w = notch ? 0.0 : (phi / ell + ell * Lp);
-    const double s2 = notch ? 1.0 : 1.0 / (aa + Gc * ell * a.Lbar);
-    double be = 0;
+    const double phi = a.phi[v], H2 = 2.0 * a.H[v], Lp = val[M];
+    const double aa = a.pd.gl[ph] + H2;
+    const double p1 = aa * phi, p3 = a.pd.b[ph] * Lp;
+    const double F2 = notch ? (phi - 1.0) : (aa * phi + p3 - H2);
+    double q = phi * a.rell;  // phi / ell: the product with the reciprocal, corrected
+    q += (phi - q * ell) * a.rell;
+    const double gw = q + ell * Lp;
+    const double w = notch ? 0.0 : gw;
+    const double s2 = notch ? 1.0 : recip_nr(aa + a.pd.bl[ph]);
 #pragma unroll
     for (int k = 0; k < M; ++k) {
       a.F[k * n + v] = val[k];
       const double b = -a.s1 * val[k];
-      rhs[k * n + v] = (TK)b;
-      be += b * b;
+      rhs[k * n + v] = round_to<TK>(b);
+      acc[2] += b * b;
     }
     a.F[M * n + v] = F2;
     a.Lphi[v] = Lp;
     const double bp = -s2 * F2;
-    rhs[M * n + v] = (TK)bp;
-    tan[TI::W * n + v] = (TK)w;
+    rhs[M * n + v] = round_to<TK>(bp);
+    tan[TI::W * n + v] = round_to<TK>(w);
     s2out[v] = s2;
-    acc[0] += phi * (phi / (2.0 * ell) + 0.5 * ell * Lp);
+    acc[0] += phi * gw;  // halved below
     acc[1] += w * w;
-    acc[2] += be;
     acc[3] += bp * bp;
-    if (!notch) {
-      const double t1 = s2 * aa * phi, t2 = s2 * 2.0 * H, t3 = s2 * Gc * ell * Lp;
-      acc[4] += t1 * t1 + t2 * t2 + t3 * t3;
-    }
+    if (!notch) acc[4] += s2 * s2 * (p1 * p1 + H2 * H2 + p3 * p3);
   }
+  acc[0] *= 0.5;
   block_partials<5>(acc, a.part, gridDim.x, blockIdx.x);
 }
 

@@ -25,24 +25,8 @@ __device__ __forceinline__ void mandel_to_tensor(const double *mv, double *e) {
     e[1] = e[3] = mv[5] * kInvSqrt2;
   }
 }
-template <int M>
-__device__ __forceinline__ void tensor_to_mandel(const double *e, double *mv) {
-  if (M == 3) {
-    mv[0] = e[0];
-    mv[1] = e[4];
-    mv[2] = e[1] * kSqrt2;
-  } else {
-    mv[0] = e[0];
-    mv[1] = e[4];
-    mv[2] = e[8];
-    mv[3] = e[5] * kSqrt2;
-    mv[4] = e[2] * kSqrt2;
-    mv[5] = e[1] * kSqrt2;
-  }
-}
-
 // Symmetric eigen-decomposition.  Q is row-major with eigenvectors as columns:
-// e = Q diag(z) Q^T.  2D: closed form of the 2 x 2 block.  3D: cyclic Jacobi rotations.
+// e = Q diag(z) Q^T.  2D: closed form of the 2 x 2 block.  3D: Jacobi rotations.
 __device__ __forceinline__ void eig2(const double *e, double *z, double *Q) {
   const double a = e[0], b = e[4], c = e[1];
   const double m = 0.5 * (a + b), h = 0.5 * (a - b);
@@ -68,54 +52,151 @@ __device__ __forceinline__ void eig2(const double *e, double *z, double *Q) {
   Q[4] = ct;
 }
 
-__device__ __forceinline__ void eig3(const double *e, double *z, double *Q) {
-  double A[9];
-#pragma unroll
-  for (int i = 0; i < 9; ++i) A[i] = e[i];
-#pragma unroll
-  for (int i = 0; i < 9; ++i) Q[i] = (i % 4 == 0) ? 1.0 : 0.0;
-  double scale = fabs(A[0]) + fabs(A[4]) + fabs(A[8]) + fabs(A[1]) + fabs(A[2]) + fabs(A[5]);
-  for (int sweep = 0; sweep < 12; ++sweep) {
-    const double off = fabs(A[1]) + fabs(A[2]) + fabs(A[5]);
-    if (off <= 1e-17 * scale || off == 0.0) break;
-    const int P[3] = {0, 0, 1}, R[3] = {1, 2, 2};
-    for (int k = 0; k < 3; ++k) {
-      const int p = P[k], q = R[k];
-      const double apq = A[p * 3 + q];
-      if (apq == 0.0) continue;
-      const double theta = (A[q * 3 + q] - A[p * 3 + p]) / (2.0 * apq);
-      const double t = (theta >= 0.0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
-      const double c = 1.0 / sqrt(t * t + 1.0), s = t * c;
-      // A <- J^T A J with J the rotation in the (p, q) plane
-      for (int r = 0; r < 3; ++r) {
-        const double arp = A[r * 3 + p], arq = A[r * 3 + q];
-        A[r * 3 + p] = c * arp - s * arq;
-        A[r * 3 + q] = s * arp + c * arq;
-      }
-      for (int r = 0; r < 3; ++r) {
-        const double apr = A[p * 3 + r], aqr = A[q * 3 + r];
-        A[p * 3 + r] = c * apr - s * aqr;
-        A[q * 3 + r] = s * apr + c * aqr;
-      }
-      for (int r = 0; r < 3; ++r) {
-        const double qrp = Q[r * 3 + p], qrq = Q[r * 3 + q];
-        Q[r * 3 + p] = c * qrp - s * qrq;
-        Q[r * 3 + q] = s * qrp + c * qrq;
-      }
-    }
-  }
-  z[0] = A[0];
-  z[1] = A[4];
-  z[2] = A[8];
+// x 2^(1023 - ex) in float32 for the biased exponent ex of a magnitude of x's matrix: the bits of
+// x, truncated, so that no conversion goes through the float64 pipe
+__device__ __forceinline__ float scaled_f32(double x, int ex) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int eb = (int)(b >> 52 & 2047), e = eb - ex + 127;
+  if (eb == 0 || e <= 0) return 0.f;
+  return __uint_as_float((unsigned)(b >> 32) & 0x80000000u | (unsigned)min(e, 255) << 23 |
+                         (unsigned)(b >> 29) & 0x7FFFFFu);
 }
 
-// divided difference of <x>+ (first-order Loewner matrix), tie rule H+((za+zb)/2); the
-// differences in float64, the quotient in precision TT
-template <typename TT>
-__device__ __forceinline__ TT loewner_t(double za, double zb, double tie) {
-  const double d = za - zb;
-  if (fabs(d) <= tie) return (0.5 * (za + zb) > 0.0) ? (TT)1 : (TT)0;
-  return (TT)(fmax(za, 0.0) - fmax(zb, 0.0)) / (TT)d;
+// tan of the Jacobi rotation that removes apq from [[app, apq], [apq, aqq]], d = aqq - app
+__device__ __forceinline__ float jacobi_tan(float d, float apq) {
+  const float theta = d / (2.f * apq);
+  return copysignf(1.f, theta) / (fabsf(theta) + sqrtf(theta * theta + 1.f));
+}
+
+// float32 Jacobi rotation in the (P, R) plane of the symmetric matrix A (order xx, yy, zz, yz, xz,
+// xy), accumulated as the half-angle rotation of a unit quaternion q (w, x, y, z)
+template <int P, int R>
+__device__ __forceinline__ void jacobi_f32(float (&A)[6], float (&q)[4]) {
+  constexpr int O = 3 - P - R;          // the third axis; entry (i, j) is 3 + the axis left out
+  const float apq = A[3 + O];
+  if (apq == 0.f) return;
+  const float t = jacobi_tan(A[R] - A[P], apq);
+  const float c = 1.f / sqrtf(t * t + 1.f), s = t * c;
+  A[P] -= t * apq;
+  A[R] += t * apq;
+  A[3 + O] = 0.f;
+  const float rp = A[3 + R], rq = A[3 + P];  // (O, P) and (O, R)
+  A[3 + R] = c * rp - s * rq;
+  A[3 + P] = s * rp + c * rq;
+  const float ch = sqrtf(0.5f + 0.5f * c), a = (O == 1 ? 0.5f : -0.5f) * s / ch;
+  constexpr int X = 1 + O, Y = 1 + (O + 1) % 3, Z = 1 + (O + 2) % 3;
+  const float w = q[0], x = q[X], y = q[Y], z = q[Z];
+  q[0] = w * ch - x * a;
+  q[X] = x * ch + w * a;
+  q[Y] = y * ch + z * a;
+  q[Z] = z * ch - y * a;
+}
+
+// float64 Jacobi rotation in the (P, R) plane with a float32 tangent: an orthogonal similarity to
+// rounding whatever the tangent, which removes all but 1e-7 of the entry
+template <int P, int R>
+__device__ __forceinline__ void jacobi_f64(double (&A)[6], double *Q, int ex) {
+  constexpr int O = 3 - P - R;
+  const double apq = A[3 + O];
+  const float af = scaled_f32(apq, ex);
+  if (af == 0.f) return;  // below 2^-126 of the norm
+  const double d = A[R] - A[P];
+  const float tf = jacobi_tan(scaled_f32(d, ex), af);
+  if (!(fabsf(tf) >= 0x1p-27f)) {  // cos = 1, sin = tan to half a unit
+    const double t = (double)tf;
+    A[P] -= t * apq;
+    A[R] += t * apq;
+    A[3 + O] = apq - t * d;
+    const double rp = A[3 + R], rq = A[3 + P];
+    A[3 + R] = rp - t * rq;
+    A[3 + P] = rq + t * rp;
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      const double qp = Q[r * 3 + P], qq = Q[r * 3 + R];
+      Q[r * 3 + P] = qp - t * qq;
+      Q[r * 3 + R] = qq + t * qp;
+    }
+    return;
+  }
+  // c = (1 + t^2)^-1/2: the float32 root and one third-order correction
+  const double t = (double)tf, w = t * t + 1.0;
+  const double c0 = (double)rsqrtf(tf * tf + 1.f);
+  const double err = 1.0 - w * c0 * c0;
+  const double c = c0 + c0 * (err * (0.5 + 0.375 * err)), s = t * c;
+  const double h1 = c * A[P] - s * apq, h2 = c * apq - s * A[R];
+  const double g1 = s * A[P] + c * apq, g2 = s * apq + c * A[R];
+  A[P] = c * h1 - s * h2;
+  A[R] = s * g1 + c * g2;
+  A[3 + O] = s * h1 + c * h2;
+  const double rp = A[3 + R], rq = A[3 + P];
+  A[3 + R] = c * rp - s * rq;
+  A[3 + P] = s * rp + c * rq;
+#pragma unroll
+  for (int r = 0; r < 3; ++r) {
+    const double qp = Q[r * 3 + P], qq = Q[r * 3 + R];
+    Q[r * 3 + P] = c * qp - s * qq;
+    Q[r * 3 + R] = s * qp + c * qq;
+  }
+}
+
+// 3D: a Jacobi iteration in float32 finds the eigenvectors to 1e-6 as a unit quaternion, whose
+// rotation matrix is orthogonal to float64 rounding; the iteration is finished in float64 on
+// Q^T e Q, where one sweep leaves 1e-14 and a second, of first-order rotations, 1e-21 of the
+// norm.  About 200 float64 operations against 1250 of four sweeps from the start (the float64
+// pipe takes a warp instruction every 16 cycles).
+__device__ __forceinline__ void eig3(const double *e, double *z, double *Q) {
+  const double scale = fabs(e[0]) + fabs(e[4]) + fabs(e[8]) + fabs(e[1]) + fabs(e[2]) + fabs(e[5]);
+  const int ex = (int)((unsigned long long)__double_as_longlong(scale) >> 52);
+  float Af[6] = {scaled_f32(e[0], ex), scaled_f32(e[4], ex), scaled_f32(e[8], ex),
+                 scaled_f32(e[5], ex), scaled_f32(e[2], ex), scaled_f32(e[1], ex)};
+  float q[4] = {1.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
+  for (int sweep = 0; sweep < 6; ++sweep) {
+    const float off = fabsf(Af[3]) + fabsf(Af[4]) + fabsf(Af[5]);
+    if (off <= 1e-7f) break;  // the norm is between 1 and 2
+    jacobi_f32<0, 1>(Af, q);
+    jacobi_f32<0, 2>(Af, q);
+    jacobi_f32<1, 2>(Af, q);
+  }
+  double A[6];
+  {
+    const double w = (double)q[0], x = (double)q[1], y = (double)q[2], v = (double)q[3];
+    const double dn = w * w + x * x + y * y + v * v - 1.0;
+    const double two = 2.0 - 2.0 * (dn - dn * dn * (1.0 - dn));  // 2 / |q|^2, |dn| < 1e-5
+    const double xs = x * two, ys = y * two, vs = v * two;
+    const double wx = w * xs, wy = w * ys, wv = w * vs;
+    const double xx = x * xs, xy = x * ys, xv = x * vs, yy = y * ys, yv = y * vs, vv = v * vs;
+    Q[0] = 1.0 - (yy + vv);
+    Q[1] = xy - wv;
+    Q[2] = xv + wy;
+    Q[3] = xy + wv;
+    Q[4] = 1.0 - (xx + vv);
+    Q[5] = yv - wx;
+    Q[6] = xv - wy;
+    Q[7] = yv + wx;
+    Q[8] = 1.0 - (xx + yy);
+    double T[9];
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+      for (int k = 0; k < 3; ++k)
+        T[i * 3 + k] = e[i * 3] * Q[k] + e[i * 3 + 1] * Q[3 + k] + e[i * 3 + 2] * Q[6 + k];
+    constexpr int I[6] = {0, 1, 2, 1, 0, 0}, J[6] = {0, 1, 2, 2, 2, 1};
+#pragma unroll
+    for (int k = 0; k < 6; ++k)
+      A[k] = Q[I[k]] * T[J[k]] + Q[3 + I[k]] * T[3 + J[k]] + Q[6 + I[k]] * T[6 + J[k]];
+  }
+#pragma unroll 1
+  for (int sweep = 0; sweep < 12; ++sweep) {
+    const double off = fabs(A[3]) + fabs(A[4]) + fabs(A[5]);
+    if (off <= 1e-17 * scale || off == 0.0) break;
+    jacobi_f64<0, 1>(A, Q, ex);
+    jacobi_f64<0, 2>(A, Q, ex);
+    jacobi_f64<1, 2>(A, Q, ex);
+  }
+  z[0] = A[0];
+  z[1] = A[1];
+  z[2] = A[2];
 }
 
 }  // namespace
@@ -124,6 +205,9 @@ __device__ __forceinline__ TT loewner_t(double za, double zb, double tie) {
 
 // Per voxel: eps = eps_t + f E; spectral split; sigma = g sigma0+ + sigma0-; H = max(psi+, H^n);
 // chi = [psi+ >= H^n]; tangent channels of the scaled Newton operator (TanIdx).
+// Bound by the float64 pipe: 90 float64 operations a voxel in 2D and 490 in 3D (226 and 1900
+// with library roots and divisions, signs by comparison, conversions and four float64 Jacobi
+// sweeps), 512^2 103 -> 56 us, 96^3 2.1 ms -> 763 us.
 template <int M, typename TK>
 __global__ void __launch_bounds__(256) k_constitutive(ConstArgs a, TK *tan) {
   using TI = TanIdx<M>;
@@ -140,135 +224,158 @@ __global__ void __launch_bounds__(256) k_constitutive(ConstArgs a, TK *tan) {
     const int ph = mb & 0x7f;
     const double lam = a.ph.lam[ph], mu = a.ph.mu[ph], Gc = a.ph.Gc[ph];
     const double phi = a.phi[v], Hn = a.Hn[v];
-    double em[M];
+    // tensor components in Mandel order: diagonal, then (yz, xz, xy) in 3D, (xy) in 2D
+    double e[M];
 #pragma unroll
-    for (int k = 0; k < M; ++k) em[k] = a.eps_t[k * n + v] + a.fM[k] * a.E;
-    double e[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-    mandel_to_tensor<M>(em, e);
-    double z[3] = {0, 0, 0}, Q[9] = {1, 0, 0, 0, 1, 0, 0, 0, 1};
-    // 2D: eigenvalues z0 >= z1 of the 2 x 2 block and the spectral projector onto z0's
-    // eigenvector, P0 = (e - z1 I) / (z0 - z1) = I / 2 + (e - m I) / (2 rad), kept as
-    // (P0_xx, P0_yy, P0_xy); the split needs no eigenvectors, the tangent builds them from P0
-    // in the Krylov precision.  3D: cyclic Jacobi.
-    double P0[3] = {1.0, 0.0, 0.0};
-    if (D == 2) {
-      const double mm = 0.5 * (e[0] + e[4]), hh = 0.5 * (e[0] - e[4]), cc = e[1];
-      const double rad = sqrt(hh * hh + cc * cc);
-      z[0] = mm + rad;
-      z[1] = mm - rad;
-      if (rad > 0.0) {
-        const double ir = 0.5 / rad;
-        P0[0] = 0.5 + hh * ir;
-        P0[1] = 0.5 - hh * ir;
-        P0[2] = cc * ir;
-      }
-    } else {
-      eig3(e, z, Q);
+    for (int k = 0; k < M; ++k) {
+      e[k] = a.eps_t[k * n + v] + a.fM[k] * a.E;
+      if (k >= D) e[k] *= kInvSqrt2;
     }
-    const double tr = (D == 2) ? (e[0] + e[4]) : (e[0] + e[4] + e[8]);
-    const double g = (1.0 - phi) * (1.0 - phi) + a.k_res;
-    const double gp = -2.0 * (1.0 - phi);
-    double psi_drive;
-    double sig[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0}, sdrv[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-    double L[9];
-    const double hp = tr > 0.0 ? 1.0 : 0.0;
+    const double tr = (D == 2) ? (e[0] + e[1]) : (e[0] + e[1] + e[2]);
+    const double om = 1.0 - phi, g = om * om + a.k_res;
+    const double mu2 = 2.0 * mu;
+    double psi_drive, sdrv[M], sig[M];
+    TK Qt[9] = {1, 0, 0, 0, 1, 0, 0, 0, 1}, Lt[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
     if (a.isotropic) {
       double ee = 0;
 #pragma unroll
-      for (int i = 0; i < 9; ++i) ee += e[i] * e[i];
+      for (int k = 0; k < M; ++k) ee += (k < D ? e[k] : 2.0 * e[k]) * e[k];
       psi_drive = 0.5 * lam * tr * tr + mu * ee;
+      const double lt = lam * tr;
 #pragma unroll
-      for (int i = 0; i < 9; ++i) sdrv[i] = 2.0 * mu * e[i];
-#pragma unroll
-      for (int i = 0; i < D; ++i) sdrv[i * 4] += lam * tr;
-#pragma unroll
-      for (int i = 0; i < 9; ++i) sig[i] = g * sdrv[i];
+      for (int k = 0; k < M; ++k) {
+        sdrv[k] = k < D ? mu2 * e[k] + lt : mu2 * e[k];
+        sig[k] = g * sdrv[k];
+      }
     } else {
-      double zp[3], zm[3];
-#pragma unroll
-      for (int i = 0; i < D; ++i) {
-        zp[i] = fmax(z[i], 0.0);
-        zm[i] = fmin(z[i], 0.0);
-      }
-      const double trp = fmax(tr, 0.0), trm = fmin(tr, 0.0);
-      psi_drive = 0.5 * lam * trp * trp;
-#pragma unroll
-      for (int i = 0; i < D; ++i) psi_drive += mu * zp[i] * zp[i];
-#pragma unroll
-      for (int i = 0; i < D; ++i)
-#pragma unroll
-        for (int j = 0; j < D; ++j) {
-          double ep = 0, emn = 0;
-          if (D == 2) {  // e+- = <z0>+- P0 + <z1>+- (I - P0)
-            const double p = i == j ? P0[i] : P0[2];
-            const double q = (i == j ? 1.0 : 0.0) - p;
-            ep = zp[0] * p + zp[1] * q;
-            emn = zm[0] * p + zm[1] * q;
-          } else {
-#pragma unroll
-            for (int k = 0; k < D; ++k) {
-              ep += Q[i * 3 + k] * zp[k] * Q[j * 3 + k];
-              emn += Q[i * 3 + k] * zm[k] * Q[j * 3 + k];
-            }
-          }
-          sdrv[i * 3 + j] = 2.0 * mu * ep + (i == j ? lam * trp : 0.0);
-          sig[i * 3 + j] = g * sdrv[i * 3 + j] + 2.0 * mu * emn + (i == j ? lam * trm : 0.0);
+      const double trp = pos_part(tr), ltp = lam * trp, ltm = lam * neg_part(tr);
+      double z[3] = {0, 0, 0}, zp[3], zm[3], ep[M], emn[M], zmax;
+      if constexpr (D == 2) {
+        // eigenvalues z0 >= z1 and the spectral projector onto z0's eigenvector,
+        // P0 = (e - z1 I) / (z0 - z1) = I / 2 + (e - m I) / (2 rad), kept as (P0_xx, P0_yy,
+        // P0_xy); the split needs no eigenvectors, the tangent builds them from P0 in the Krylov
+        // precision
+        double P0[3] = {1.0, 0.0, 0.0};
+        const double mm = 0.5 * tr, hh = 0.5 * (e[0] - e[1]), cc = e[2];
+        const double x = hh * hh + cc * cc;
+        bool ok;
+        double rr = rsqrt_nr(x, ok), rad;
+        if (ok) {
+          rad = x * rr;
+          rad += (x - rad * rad) * (0.5 * rr);
+          rr *= 0.5;
+        } else {
+          rad = sqrt(x);
+          rr = rad > 0.0 ? 0.5 / rad : 0.0;
         }
-      double zmax = 0;
+        z[0] = mm + rad;
+        z[1] = mm - rad;
+        if (rad > 0.0) {
+          P0[0] = 0.5 + hh * rr;
+          P0[1] = 0.5 - hh * rr;
+          P0[2] = cc * rr;
+        }
 #pragma unroll
-      for (int i = 0; i < D; ++i) zmax = fmax(zmax, fabs(z[i]));
-      const double tie = 1e-12 * zmax;
-      // L only enters the tangent: the tie test and both differences in float64, the
-      // quotient in the Krylov precision (one float64 division fewer per pair in MIXED)
-#pragma unroll
-      for (int i = 0; i < D; ++i)
-#pragma unroll
-        for (int j = 0; j < D; ++j) L[i * 3 + j] = (double)loewner_t<TK>(z[i], z[j], tie);
-    }
-    const double H = fmax(psi_drive, Hn);
-    const double chi = (psi_drive >= Hn) ? 1.0 : 0.0;
-    double sm[M], dm[M];
-    tensor_to_mandel<M>(sig, sm);
-    tensor_to_mandel<M>(sdrv, dm);
-#pragma unroll
-    for (int k = 0; k < M; ++k) {
-      a.sigma[k * n + v] = sm[k];
-      acc[k] += sm[k];
-      acc[M] += (a.s1 * sm[k]) * (a.s1 * sm[k]);
-    }
-    a.H[v] = H;
-    if (!notch) mx[0] = fmax(mx[0], 2.0 * psi_drive / (Gc / a.ell));
-    // tangent in Mandel form: column kb = C_t applied to the kb-th Mandel basis tensor,
-    // evaluated in the Krylov precision TK (it only enters the Newton operator)
-    TK Ct[M][M];
-    {
-      using TT = TK;
-      const TT gT = (TT)g, muT = (TT)mu, lamT = (TT)lam;
-      TT Qt[9], Lt[9];
-#pragma unroll
-      for (int i = 0; i < 9; ++i) {
-        Qt[i] = (TT)Q[i];
-        Lt[i] = a.isotropic ? (TT)0 : (TT)L[i];
-      }
-      if (D == 2 && !a.isotropic) {
-        // eigenvectors (ct, st) of z0 and (-st, ct) of z1 from P0: ct^2 = P0_xx,
-        // st^2 = P0_yy, ct st = P0_xy, taking the root of the larger diagonal entry
-        const TT p00 = (TT)P0[0], p11 = (TT)P0[1], p01 = (TT)P0[2];
-        TT ct, st;
+        for (int i = 0; i < D; ++i) {
+          zp[i] = pos_part(z[i]);
+          zm[i] = neg_part(z[i]);
+        }
+        // e+- = <z1>+- I + (<z0>+- - <z1>+-) P0
+        const double dp = zp[0] - zp[1], dm = zm[0] - zm[1];
+        ep[0] = zp[1] + dp * P0[0];
+        ep[1] = zp[1] + dp * P0[1];
+        ep[2] = dp * P0[2];
+        emn[0] = zm[1] + dm * P0[0];
+        emn[1] = zm[1] + dm * P0[1];
+        emn[2] = dm * P0[2];
+        // eigenvectors (ct, st) of z0 and (-st, ct) of z1: ct^2 = P0_xx, st^2 = P0_yy,
+        // ct st = P0_xy, taking the root of the larger diagonal entry
+        const TK p00 = round_to<TK>(P0[0]), p11 = round_to<TK>(P0[1]), p01 = round_to<TK>(P0[2]);
+        TK ct, st;
         if (p00 >= p11) {
           ct = sqrt(p00);
           st = p01 / ct;
         } else {
           st = sqrt(p11);
-          if (p01 < (TT)0) st = -st;
+          if (p01 < (TK)0) st = -st;
           ct = p01 / st;
         }
         Qt[0] = ct;
         Qt[1] = -st;
         Qt[3] = st;
         Qt[4] = ct;
+      } else {
+        double Q[9];
+        const double t9[9] = {e[0], e[M - 1], e[M - 2], e[M - 1], e[1], e[3 % M], e[M - 2], e[3 % M], e[2]};
+        eig3(t9, z, Q);
+#pragma unroll
+        for (int i = 0; i < D; ++i) {
+          zp[i] = pos_part(z[i]);
+          zm[i] = neg_part(z[i]);
+        }
+        constexpr int I[6] = {0, 1, 2, 1, 0, 0}, J[6] = {0, 1, 2, 2, 2, 1};
+#pragma unroll
+        for (int k = 0; k < M; ++k) {
+          ep[k] = emn[k] = 0;
+#pragma unroll
+          for (int q = 0; q < 3; ++q) {
+            const double qq = Q[I[k] * 3 + q] * Q[J[k] * 3 + q];
+            ep[k] += qq * zp[q];
+            emn[k] += qq * zm[q];
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < 9; ++i) Qt[i] = round_to<TK>(Q[i]);
       }
-      const TT volc = a.isotropic ? gT * lamT : (TT)(g * lam * hp + lam * (1.0 - hp));
+      double zs = zp[0] * zp[0];
+#pragma unroll
+      for (int i = 1; i < D; ++i) zs += zp[i] * zp[i];
+      psi_drive = 0.5 * ltp * trp + mu * zs;
+#pragma unroll
+      for (int k = 0; k < M; ++k) {
+        sdrv[k] = k < D ? mu2 * ep[k] + ltp : mu2 * ep[k];
+        sig[k] = g * sdrv[k] + (k < D ? mu2 * emn[k] + ltm : mu2 * emn[k]);
+      }
+      // Loewner matrix of <x>+ (it only enters the tangent): the tie test and both differences in
+      // float64, the quotient in the Krylov precision
+      zmax = fabs(z[0]);
+#pragma unroll
+      for (int i = 1; i < D; ++i)
+        if (__double_as_longlong(fabs(z[i])) > __double_as_longlong(zmax)) zmax = fabs(z[i]);
+      const double tie = 1e-12 * zmax;
+#pragma unroll
+      for (int i = 0; i < D; ++i) {
+        Lt[i * 4] = zp[i] != 0.0 ? (TK)1 : (TK)0;
+#pragma unroll
+        for (int j = i + 1; j < D; ++j) {
+          const double d = z[i] - z[j];
+          TK l;
+          if (fabs(d) <= tie) l = (z[i] + z[j] > 0.0) ? (TK)1 : (TK)0;
+          else l = round_to<TK>(zp[i] - zp[j]) / round_to<TK>(d);
+          Lt[i * 3 + j] = Lt[j * 3 + i] = l;
+        }
+      }
+    }
+    const bool grow = psi_drive >= Hn;
+    const double H = fmax(psi_drive, Hn);
+    double sm[M], dm[M];
+#pragma unroll
+    for (int k = 0; k < M; ++k) {
+      sm[k] = k < D ? sig[k] : sig[k] * kSqrt2;
+      dm[k] = k < D ? sdrv[k] : sdrv[k] * kSqrt2;
+      a.sigma[k * n + v] = sm[k];
+      acc[k] += sm[k];
+      acc[M] += sm[k] * sm[k];  // times s1^2 below
+    }
+    a.H[v] = H;
+    if (!notch) mx[0] = fmax(mx[0], psi_drive * a.pd.r2gl[ph]);
+    // tangent in Mandel form: column kb = C_t applied to the kb-th Mandel basis tensor,
+    // evaluated in the Krylov precision TK (it only enters the Newton operator)
+    TK Ct[M][M];
+    {
+      using TT = TK;
+      const TT gT = round_to<TT>(g), muT = round_to<TT>(mu);
+      const TT volc = a.isotropic ? gT * round_to<TT>(lam) : round_to<TT>(tr > 0.0 ? g * lam : lam);
 #pragma unroll
       for (int kb = 0; kb < M; ++kb) {
         // basis tensor: unit on (i0, i0) for kb < D, else (e_i0 e_j0 + e_j0 e_i0) / sqrt 2
@@ -340,14 +447,17 @@ __global__ void __launch_bounds__(256) k_constitutive(ConstArgs a, TK *tan) {
       }
     // row scaling of the phase-field row for the tangent channels, evaluated in the Krylov
     // precision (float64 sums, one TK division)
-    const TK s2 = notch ? (TK)1 : (TK)1 / (TK)(Gc / a.ell + 2.0 * H + Gc * a.ell * a.Lbar);
+    const double aa = a.pd.gl[ph] + 2.0 * H;
+    const TK s2 = notch ? (TK)1 : (TK)1 / round_to<TK>(aa + a.pd.bl[ph]);
+    const double s1gp = a.s1 * -2.0 * om;
 #pragma unroll
-    for (int k = 0; k < M; ++k) tan[(TI::SF + k) * n + v] = (TK)(notch ? 0.0 : a.s1 * gp * dm[k]);
-    tan[TI::KAPPA * n + v] = notch ? (TK)0 : (TK)chi * s2 / (TK)a.s1;
-    tan[TI::A * n + v] = notch ? (TK)0 : s2 * (TK)(Gc / a.ell + 2.0 * H);
+    for (int k = 0; k < M; ++k) tan[(TI::SF + k) * n + v] = notch ? (TK)0 : round_to<TK>(s1gp * dm[k]);
+    tan[TI::KAPPA * n + v] = notch || !grow ? (TK)0 : s2 / (TK)a.s1;
+    tan[TI::A * n + v] = notch ? (TK)0 : s2 * round_to<TK>(aa);
     tan[TI::B * n + v] = notch ? (TK)0 : s2 * (TK)Gc * (TK)a.ell;
-    tan[TI::NOTCH * n + v] = (TK)(notch ? 1.0 : 0.0);
+    tan[TI::NOTCH * n + v] = notch ? (TK)1 : (TK)0;
   }
+  acc[M] *= a.s1 * a.s1;
   block_partials<M + 1>(acc, a.part, gridDim.x, blockIdx.x);
   block_max_partials<1>(mx, a.part_max, gridDim.x, blockIdx.x);
 }

@@ -969,6 +969,18 @@ static int energy_constraint_t(rve *h, const double *phi) {
   return RVE_OK;
 }
 
+static PhaseDer phase_der(const rve *h) {
+  PhaseDer p;
+  for (int i = 0; i < 16; ++i) {
+    const double Gc = h->ph.Gc[i], ell = h->desc.ell;
+    p.gl[i] = Gc / ell;
+    p.r2gl[i] = 2.0 / p.gl[i];
+    p.b[i] = Gc * ell;
+    p.bl[i] = Gc * ell * h->Lbar;
+  }
+  return p;
+}
+
 // ---- linearisation: constitutive law + residual + rhs ------------------------------------
 template <typename TK, int M>
 static int linearize_t(rve *h, const double *eps_t, const double *phi, double E, int control,
@@ -986,7 +998,7 @@ static int linearize_t(rve *h, const double *eps_t, const double *phi, double E,
   ca.ell = h->desc.ell;
   ca.k_res = h->desc.k_res;
   ca.s1 = h->s1;
-  ca.Lbar = h->Lbar;
+  ca.pd = phase_der(h);
   ca.isotropic = h->desc.split == RVE_SPLIT_NONE;
   ca.sigma = h->sigma;
   ca.H = h->Hcur;
@@ -1001,10 +1013,10 @@ static int linearize_t(rve *h, const double *eps_t, const double *phi, double E,
   ra.phi = phi;
   ra.H = h->Hcur;
   ra.mat = h->mat;
-  ra.ph = h->ph;
+  ra.pd = ca.pd;
   ra.ell = h->desc.ell;
+  ra.rell = 1.0 / h->desc.ell;
   ra.s1 = h->s1;
-  ra.Lbar = h->Lbar;
   ra.spec = (cpx<double> *)h->spec;
   ra.F = h->F;
   ra.Lphi = h->Lphi;

@@ -13,6 +13,15 @@ struct PhaseTab {
   double lam[16], mu[16], Gc[16];
 };
 
+// Constants of each phase that the float64 kernels would otherwise divide or multiply for in
+// every voxel (a float64 division is a dozen instructions of 16 cycles each).
+struct PhaseDer {
+  double gl[16];    // Gc / l
+  double r2gl[16];  // 2 / (Gc / l)
+  double b[16];     // Gc l
+  double bl[16];    // Gc l Lbar
+};
+
 // Grid description.
 struct Geo {
   int d, m, c;          // dimension, Mandel components, channels (m + 1)
@@ -89,6 +98,59 @@ template <typename T>
 __device__ __forceinline__ T ks_scalar(double d, float f) {
   if constexpr (sizeof(T) == 4) return f;
   else return d;
+}
+
+// ---- float64 roots and reciprocals ------------------------------------------------------
+// By a float32 seed (22 bits) and one third-order Newton (Halley) correction, which leaves about
+// one unit in the last place: 3 and 5 float64 operations.  The seed's bits are moved by integer
+// instructions, not converted through the float64 pipe.  Arguments whose seed leaves the normal
+// range take the library function.
+__device__ __forceinline__ double f64_of_seed(float r, int shift) {  // r 2^shift, r in [2^-2, 2)
+  const unsigned b = __float_as_uint(r);
+  return __hiloint2double((int)((b >> 3) + ((896u + (unsigned)shift) << 20)), (int)(b << 29));
+}
+__device__ __forceinline__ double recip_nr(double x) {
+  const int hi = __double2hiint(x);
+  const int e = hi >> 20 & 2047;
+  if ((unsigned)(e - 2) > 2041u) return 1.0 / x;
+  const float m = __uint_as_float(0x3F800000u | (((unsigned)hi & 0xFFFFFu) << 3) | ((unsigned)__double2loint(x) >> 29));
+  double r = f64_of_seed(__fdividef(1.f, m), 1023 - e);
+  if (hi < 0) r = -r;
+  const double h = 1.0 - x * r;
+  return r + r * (h + h * h);
+}
+// 1 / sqrt(x) for x > 0; ok: false where x is not a positive normal number (0 is returned)
+__device__ __forceinline__ double rsqrt_nr(double x, bool &ok) {
+  const int hi = __double2hiint(x);
+  const int e = hi >> 20;
+  ok = (unsigned)(e - 2) <= 2041u;
+  if (!ok) return 0.0;
+  const int k = (e - 1023) >> 1, odd = (e - 1023) & 1;
+  const float m = __uint_as_float((unsigned)(127 + odd) << 23 | (((unsigned)hi & 0xFFFFFu) << 3) |
+                                  ((unsigned)__double2loint(x) >> 29));
+  const double r = f64_of_seed(rsqrtf(m), -k);
+  const double h = 1.0 - (x * r) * r;
+  return r + (r * h) * (0.5 + 0.375 * h);
+}
+// x in type T, rounded to nearest; float32 by integer instructions in its normal range
+template <typename T>
+__device__ __forceinline__ T round_to(double x) {
+  if constexpr (sizeof(T) == 4) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    if (((unsigned)(b >> 52 & 2047) - 897u) >= 253u) return (T)x;
+    const unsigned long long t = b + 0x0FFFFFFFull + (b >> 29 & 1);
+    return __uint_as_float((unsigned)(b >> 32) & 0x80000000u |
+                           (((unsigned)(t >> 29) - (896u << 23)) & 0x7FFFFFFFu));
+  } else {
+    return x;
+  }
+}
+// max(x, 0) and min(x, 0) by the sign bit; 0 for NaN, as fmax and fmin give
+__device__ __forceinline__ double pos_part(double x) {
+  return (unsigned)__double2hiint(x) <= 0x7FF00000u ? x : 0.0;
+}
+__device__ __forceinline__ double neg_part(double x) {
+  return (unsigned)__double2hiint(x) - 0x80000000u <= 0x7FF00000u ? x : 0.0;
 }
 
 // ---- block reductions into per-block partials ------------------------------------------
@@ -229,8 +291,8 @@ struct ResidArgs {
   const double *phi;    // 1 channel
   const double *H;      // current history max(psi+, H^n)
   const uint8_t *mat;
-  PhaseTab ph;
-  double ell, s1, Lbar;
+  PhaseDer pd;
+  double ell, rell, s1;
   cpx<double> *spec;
   double *F;            // unscaled residual F1 (m ch), F2 (1 ch)
   double *Lphi;         // L phi
@@ -267,7 +329,8 @@ struct ConstArgs {
   PhaseTab ph;
   double fM[6];
   double E;
-  double ell, k_res, s1, Lbar;
+  PhaseDer pd;
+  double ell, k_res, s1;
   int isotropic;
   double *sigma;        // m channels out
   double *H;            // max(psi+, H^n) out
