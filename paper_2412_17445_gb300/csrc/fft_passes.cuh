@@ -661,10 +661,25 @@ __global__ void __launch_bounds__(256) k_xinv_apply(const __grid_constant__ Appl
   extern __shared__ unsigned char smraw[];
   cpx<T> *sm = reinterpret_cast<cpx<T> *>(smraw);
   if (a.ks && a.ks->done) return;
+  // fin 3, 4: block 0 only forms the E slot of y, from the constraint-row partials of the x-forward
+  // pass (an earlier launch), while the others run the pass: the chain of the 128-bit sum takes
+  // 4 us, a quarter of the pass at 512^2
+  const bool yE_block = a.fin == 3 || a.fin == 4;
+  const int G = (int)gridDim.x - (yE_block ? 1 : 0);
+  const int blk = (int)blockIdx.x - (yE_block ? 1 : 0);
+  if (blk < 0) {
+    if (a.fin == 4) {
+      if (threadIdx.x == 0) *a.yE = *a.xE_ptr;
+    } else if (threadIdx.x < 32) {
+      const double sE = warp_sum_exact<false>(a.part, G);
+      if (threadIdx.x == 0) *a.yE = sE;
+    }
+    return;
+  }
   const Geo &g = a.g;
   const int c = M + 1, nx = NL > 0 ? NL : g.nx, Np = line_slots<NL>(pl.Np);
   const int n = (int)g.n;
-  const int row0 = blockIdx.x * 2 * P;
+  const int row0 = blk * 2 * P;
   const FDiv dnx = make_fdiv(nx);
   xinv_head<T, NL>(sm, c, P, row0, g, pl, a.spec, a.tr);
   [[maybe_unused]] const unsigned long long *meta = nullptr;
@@ -691,25 +706,19 @@ __global__ void __launch_bounds__(256) k_xinv_apply(const __grid_constant__ Appl
     if (ok1) epi_compute<T, M>(a, n, v1, y1, in1, d, em);
   }
   if (em == 6) {
-    block_partials_k<T, 5>(d, a.part + gridDim.x, gridDim.x, blockIdx.x);
+    block_partials_k<T, 5>(d, a.part + G, G, blk);
   } else if (em != 0) {
     const T pv[2] = {d[0], d[1]};
-    block_partials_k<T, 2>(pv, a.part + gridDim.x, gridDim.x, blockIdx.x);
+    block_partials_k<T, 2>(pv, a.part + G, G, blk);
   }
   if (a.fin == 1 || a.fin == 2 || a.fin == 5 || a.fin == 6) {
     // the member's last block finalises the iteration's scalars (no separate launch)
-    if (last_block_arrives(a.arrive, gridDim.x)) {
-      if (a.fin == 1) fin_alpha<true>(a.ksw, a.part, gridDim.x);
-      else if (a.fin == 2) fin_omega<true>(a.ksw, a.part, gridDim.x);
-      else if (a.fin == 5) fin_alpha_clear<true>(a.ksw, a.part, gridDim.x);
-      else fin_omega_conv<true>(a.ksw, a.part, gridDim.x);
+    if (last_block_arrives(a.arrive, G)) {
+      if (a.fin == 1) fin_alpha<true>(a.ksw, a.part, G);
+      else if (a.fin == 2) fin_omega<true>(a.ksw, a.part, G);
+      else if (a.fin == 5) fin_alpha_clear<true>(a.ksw, a.part, G);
+      else fin_omega_conv<true>(a.ksw, a.part, G);
     }
-  } else if (a.fin == 3 && blockIdx.x == 0 && threadIdx.x < 32) {
-    // the constraint-row partials come from the x-forward pass (an earlier launch)
-    const double sE = warp_sum_exact<false>(a.part, gridDim.x);
-    if (threadIdx.x == 0) *a.yE = sE;
-  } else if (a.fin == 4 && blockIdx.x == 0 && threadIdx.x == 0) {
-    *a.yE = *a.xE_ptr;
   }
 }
 

@@ -839,7 +839,8 @@ static int apply_scaled(rve *h, TK *x, const double *xE_ptr, TK *y, int pro_mode
   CKL();
   TRY((launch_columns<TK, M>(h, a.spec, ks, dbl ? h->Wy_d : h->Wy, dbl ? h->Wz_d : h->Wz,
                              dbl ? h->smy_d : h->smy_k, dbl ? h->smz_d : h->smz_k)));
-  row_kernel<TK, M, false>(ct_len(h, 0), P, a.epi_mode)<<<Gx, 256, smx, h->stream>>>(solo(a), plan_of<TK>(h, 0), P);
+  // fin 3, 4: one more block for the E slot
+  row_kernel<TK, M, false>(ct_len(h, 0), P, a.epi_mode)<<<Gx + (yE ? 1 : 0), 256, smx, h->stream>>>(solo(a), plan_of<TK>(h, 0), P);
   h->launches += 1;
   CKL();
   return RVE_OK;
@@ -2928,7 +2929,8 @@ static int apply_batch_t(rve *const *hs, int n, const void *const *x, const doub
   CKL();
   TRY((launch_columns_n<TK, M>(h, spec, ks, n, dbl ? h->Wy_d : h->Wy, dbl ? h->Wz_d : h->Wz,
                                dbl ? h->smy_d : h->smy_k, dbl ? h->smz_d : h->smz_k, st)));
-  row_kernel<TK, M, false>(ct_len(h, 0), P, A.m[0].epi_mode)<<<gx, 256, smx, st>>>(A, plan_of<TK>(h, 0), P);
+  const dim3 gi(Gx + 1, n);  // one more block a member for the E slot
+  row_kernel<TK, M, false>(ct_len(h, 0), P, A.m[0].epi_mode)<<<gi, 256, smx, st>>>(A, plan_of<TK>(h, 0), P);
   h->launches += 1;
   CKL();
   return RVE_OK;

@@ -274,8 +274,8 @@ struct ApplyArgs {
   const KrylovScalars *ks;
   int tr;               // 1: spectral scratch transposed [ch][kx][row] (fused 2D column pass)
   // finalisation by the x-inverse pass itself (krylov_fin.cuh): 0 none; 1 / 2 the member's
-  // last block runs the alpha / omega update on ksw (epilogue modes 1 / 2); 3 block 0 writes
-  // yE = sum of the constraint-row partials; 4 block 0 copies *xE_ptr to yE (strain control);
+  // last block runs the alpha / omega update on ksw (epilogue modes 1 / 2); 3 one more block, the
+  // first, writes yE = sum of the constraint-row partials; 4 it copies *xE_ptr to yE (strain control);
   // 5 the last block runs the alpha update and clears ks->pending; 6 the last block runs the
   // merged omega / convergence update (epilogue mode 6) and sets ks->pending
   int fin;
