@@ -118,16 +118,23 @@ __device__ __forceinline__ void jacobi_f64(double (&A)[6], double *Q, int ex) {
     }
     return;
   }
-  // c = (1 + t^2)^-1/2: the float32 root and one third-order correction
-  const double t = (double)tf, w = t * t + 1.0;
-  const double c0 = (double)rsqrtf(tf * tf + 1.f);
-  const double err = 1.0 - w * c0 * c0;
-  const double c = c0 + c0 * (err * (0.5 + 0.375 * err)), s = t * c;
-  const double h1 = c * A[P] - s * apq, h2 = c * apq - s * A[R];
-  const double g1 = s * A[P] + c * apq, g2 = s * apq + c * A[R];
-  A[P] = c * h1 - s * h2;
-  A[R] = s * g1 + c * g2;
-  A[3 + O] = s * h1 + c * h2;
+  // c = (1 + t^2)^-1/2: two terms of the series below 1e-4 (the third is 4e-17), else the float32
+  // root and one third-order correction
+  const double t = (double)tf, t2 = t * t;
+  const double left = apq - t * d;  // what the float32 tangent leaves, over c^2
+  double c, rest = left - t2 * apq;
+  if (fabsf(tf) < 1e-4f) {
+    c = 1.0 - 0.5 * t2;
+  } else {
+    const double c0 = (double)rsqrtf(tf * tf + 1.f);
+    const double err = 1.0 - (t2 + 1.0) * c0 * c0;
+    c = c0 + c0 * (err * (0.5 + 0.375 * err));
+    rest *= c * c;
+  }
+  const double s = t * c, move = s * c * (apq + left);
+  A[P] -= move;
+  A[R] += move;
+  A[3 + O] = rest;
   const double rp = A[3 + R], rq = A[3 + P];
   A[3 + R] = c * rp - s * rq;
   A[3 + P] = s * rp + c * rq;
@@ -205,9 +212,9 @@ __device__ __forceinline__ void eig3(const double *e, double *z, double *Q) {
 
 // Per voxel: eps = eps_t + f E; spectral split; sigma = g sigma0+ + sigma0-; H = max(psi+, H^n);
 // chi = [psi+ >= H^n]; tangent channels of the scaled Newton operator (TanIdx).
-// Bound by the float64 pipe: 90 float64 operations a voxel in 2D and 490 in 3D (226 and 1900
+// Bound by the float64 pipe: 100 float64 operations a voxel in 2D and 430 in 3D (226 and 1900
 // with library roots and divisions, signs by comparison, conversions and four float64 Jacobi
-// sweeps), 512^2 103 -> 56 us, 96^3 2.1 ms -> 763 us.
+// sweeps), 512^2 103 -> 56 us, 96^3 2.1 ms -> 700 us.
 template <int M, typename TK>
 __global__ void __launch_bounds__(256) k_constitutive(ConstArgs a, TK *tan) {
   using TI = TanIdx<M>;
@@ -249,7 +256,18 @@ __global__ void __launch_bounds__(256) k_constitutive(ConstArgs a, TK *tan) {
       }
     } else {
       const double trp = pos_part(tr), ltp = lam * trp, ltm = lam * neg_part(tr);
-      double z[3] = {0, 0, 0}, zp[3], zm[3], ep[M], emn[M], zmax;
+      double z[3] = {0, 0, 0}, zp[3], zmax;
+      // eigenvalues' weights in the driving stress (2 mu <z>+) and in the stress (that times g, and
+      // 2 mu <z>-)
+      double ws[3], wg[3];
+      auto weigh = [&]() {
+#pragma unroll
+        for (int i = 0; i < D; ++i) {
+          zp[i] = pos_part(z[i]);
+          ws[i] = mu2 * zp[i];
+          wg[i] = __double2hiint(zp[i]) != 0 ? g * ws[i] : mu2 * neg_part(z[i]);
+        }
+      };
       if constexpr (D == 2) {
         // eigenvalues z0 >= z1 and the spectral projector onto z0's eigenvector,
         // P0 = (e - z1 I) / (z0 - z1) = I / 2 + (e - m I) / (2 rad), kept as (P0_xx, P0_yy,
@@ -275,19 +293,14 @@ __global__ void __launch_bounds__(256) k_constitutive(ConstArgs a, TK *tan) {
           P0[1] = 0.5 - hh * rr;
           P0[2] = cc * rr;
         }
+        weigh();
+        // drive and stress = w1 I + (w0 - w1) P0
+        const double ds = ws[0] - ws[1], dg = wg[0] - wg[1];
 #pragma unroll
-        for (int i = 0; i < D; ++i) {
-          zp[i] = pos_part(z[i]);
-          zm[i] = neg_part(z[i]);
+        for (int k = 0; k < M; ++k) {
+          sdrv[k] = ds * P0[k] + (k < D ? ws[1] : 0.0);
+          sig[k] = dg * P0[k] + (k < D ? wg[1] : 0.0);
         }
-        // e+- = <z1>+- I + (<z0>+- - <z1>+-) P0
-        const double dp = zp[0] - zp[1], dm = zm[0] - zm[1];
-        ep[0] = zp[1] + dp * P0[0];
-        ep[1] = zp[1] + dp * P0[1];
-        ep[2] = dp * P0[2];
-        emn[0] = zm[1] + dm * P0[0];
-        emn[1] = zm[1] + dm * P0[1];
-        emn[2] = dm * P0[2];
         // eigenvectors (ct, st) of z0 and (-st, ct) of z1: ct^2 = P0_xx, st^2 = P0_yy,
         // ct st = P0_xy, taking the root of the larger diagonal entry
         const TK p00 = round_to<TK>(P0[0]), p11 = round_to<TK>(P0[1]), p01 = round_to<TK>(P0[2]);
@@ -308,20 +321,16 @@ __global__ void __launch_bounds__(256) k_constitutive(ConstArgs a, TK *tan) {
         double Q[9];
         const double t9[9] = {e[0], e[M - 1], e[M - 2], e[M - 1], e[1], e[3 % M], e[M - 2], e[3 % M], e[2]};
         eig3(t9, z, Q);
-#pragma unroll
-        for (int i = 0; i < D; ++i) {
-          zp[i] = pos_part(z[i]);
-          zm[i] = neg_part(z[i]);
-        }
+        weigh();
         constexpr int I[6] = {0, 1, 2, 1, 0, 0}, J[6] = {0, 1, 2, 2, 2, 1};
 #pragma unroll
         for (int k = 0; k < M; ++k) {
-          ep[k] = emn[k] = 0;
+          sdrv[k] = sig[k] = 0;
 #pragma unroll
           for (int q = 0; q < 3; ++q) {
             const double qq = Q[I[k] * 3 + q] * Q[J[k] * 3 + q];
-            ep[k] += qq * zp[q];
-            emn[k] += qq * zm[q];
+            sdrv[k] += qq * ws[q];
+            sig[k] += qq * wg[q];
           }
         }
 #pragma unroll
@@ -331,10 +340,11 @@ __global__ void __launch_bounds__(256) k_constitutive(ConstArgs a, TK *tan) {
 #pragma unroll
       for (int i = 1; i < D; ++i) zs += zp[i] * zp[i];
       psi_drive = 0.5 * ltp * trp + mu * zs;
+      const double vol = g * ltp + ltm;
 #pragma unroll
-      for (int k = 0; k < M; ++k) {
-        sdrv[k] = k < D ? mu2 * ep[k] + ltp : mu2 * ep[k];
-        sig[k] = g * sdrv[k] + (k < D ? mu2 * emn[k] + ltm : mu2 * emn[k]);
+      for (int k = 0; k < D; ++k) {
+        sdrv[k] += ltp;
+        sig[k] += vol;
       }
       // Loewner matrix of <x>+ (it only enters the tangent): the tie test and both differences in
       // float64, the quotient in the Krylov precision
@@ -345,7 +355,7 @@ __global__ void __launch_bounds__(256) k_constitutive(ConstArgs a, TK *tan) {
       const double tie = 1e-12 * zmax;
 #pragma unroll
       for (int i = 0; i < D; ++i) {
-        Lt[i * 4] = zp[i] != 0.0 ? (TK)1 : (TK)0;
+        Lt[i * 4] = __double2hiint(zp[i]) != 0 ? (TK)1 : (TK)0;
 #pragma unroll
         for (int j = i + 1; j < D; ++j) {
           const double d = z[i] - z[j];
