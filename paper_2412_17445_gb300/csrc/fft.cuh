@@ -296,6 +296,88 @@ __device__ __forceinline__ void fft_stage_r(cpx<T> *sm, const LineLayout &ly, co
   }
 }
 
+// Stages s and s - 1, both of radix 3, in one step: nine elements of a thread, the operations of the
+// two stages in their order (forward: s first; inverse: s - 1 first), one barrier instead of two.
+// Float32 only: fixed-point values would take 126 registers of the residual passes' 80.
+// 243 x 729 float32 apply 49.2 -> 43.2 us.
+template <typename T, bool DIT>
+__device__ __forceinline__ void fft_stage_33(cpx<T> *sm, const LineLayout &ly, const FftPlan &pl, int s) {
+  using Tw = typename FftTypes<T>::Tw;
+  using Dir = typename FftTypes<T>::Dir;
+  const Dir dir = DIT ? 1 : -1;
+  const int N = pl.N, Ns = pl.Ns[s - 1];
+  const int nb = N / 9;
+  const int tot = ly.L * nb;
+  const int twB = N / (Ns * 3), twA = N / (Ns * 9);
+  const Tw *tw = (const Tw *)pl.tw;
+  FDiv dnb;
+  dnb.d = nb;
+  dnb.m = nb > 1 ? (0xFFFFFFFFu / (unsigned)nb) + 1u : 0u;
+  for (int b = threadIdx.x; b < tot; b += blockDim.x) {
+    int l, q;
+    if (ly.line_fastest) {
+      q = (int)fdiv((unsigned)b, ly.dL);
+      l = b - q * ly.L;
+    } else {
+      l = (int)fdiv((unsigned)b, dnb);
+      q = b - l * nb;
+    }
+    const int g = (int)fdiv((unsigned)q, pl.dNs[s - 1]);
+    const int j = q - g * Ns;
+    const int e0 = g * Ns * 9 + j;
+    const int lb = line_base(ly, l);
+    cpx<T> v[3][3];  // v[k][r]: element e0 + (3 k + r) Ns
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+      for (int r = 0; r < 3; ++r) v[k][r] = sm[lb + pad8(e0 + (3 * k + r) * Ns) * ly.es];
+    auto outer = [&]() {
+#pragma unroll
+      for (int r = 0; r < 3; ++r) {
+        cpx<T> u[3] = {v[0][r], v[1][r], v[2][r]};
+        const int jt = (j + r * Ns) * twA;
+        if (DIT && jt != 0) {
+          u[1] = cmul_conj(u[1], tw[jt]);
+          u[2] = cmul_conj(u[2], tw[2 * jt]);
+        }
+        dft3(u, dir);
+        if (!DIT && jt != 0) {
+          u[1] = cmul(u[1], tw[jt]);
+          u[2] = cmul(u[2], tw[2 * jt]);
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) v[k][r] = u[k];
+      }
+    };
+    auto inner = [&]() {
+      const int jt = j * twB;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        if (DIT && jt != 0) {
+          v[k][1] = cmul_conj(v[k][1], tw[jt]);
+          v[k][2] = cmul_conj(v[k][2], tw[2 * jt]);
+        }
+        dft3(v[k], dir);
+        if (!DIT && jt != 0) {
+          v[k][1] = cmul(v[k][1], tw[jt]);
+          v[k][2] = cmul(v[k][2], tw[2 * jt]);
+        }
+      }
+    };
+    if (DIT) {
+      inner();
+      outer();
+    } else {
+      outer();
+      inner();
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+      for (int r = 0; r < 3; ++r) sm[lb + pad8(e0 + (3 * k + r) * Ns) * ly.es] = v[k][r];
+  }
+}
+
 template <typename T, bool DIT>
 __device__ __forceinline__ void fft_stage(cpx<T> *sm, const LineLayout &ly, const FftPlan &pl, int s,
                                           typename FftTypes<T>::Dir dir, const unsigned long long *meta) {
@@ -312,7 +394,14 @@ __device__ __forceinline__ void fft_stage(cpx<T> *sm, const LineLayout &ly, cons
 template <typename T>
 __device__ void fft_dif(cpx<T> *sm, const LineLayout &ly, const FftPlan &pl, const unsigned long long *meta = nullptr) {
   for (int s = pl.S - 1; s >= 0; --s) {
-    fft_stage<T, false>(sm, ly, pl, s, -1, meta);
+    bool two = false;
+    if constexpr (!FftTypes<T>::kFixed) two = s > 0 && pl.R[s] == 3 && pl.R[s - 1] == 3;
+    if (two) {
+      if constexpr (!FftTypes<T>::kFixed) fft_stage_33<T, false>(sm, ly, pl, s);
+      --s;
+    } else {
+      fft_stage<T, false>(sm, ly, pl, s, -1, meta);
+    }
     __syncthreads();
   }
 }
@@ -320,14 +409,23 @@ __device__ void fft_dif(cpx<T> *sm, const LineLayout &ly, const FftPlan &pl, con
 template <typename T>
 __device__ void fft_dit(cpx<T> *sm, const LineLayout &ly, const FftPlan &pl, const unsigned long long *meta = nullptr) {
   for (int s = 0; s < pl.S; ++s) {
-    fft_stage<T, true>(sm, ly, pl, s, 1, meta);
+    bool two = false;
+    if constexpr (!FftTypes<T>::kFixed) two = s + 1 < pl.S && pl.R[s] == 3 && pl.R[s + 1] == 3;
+    if (two) {
+      ++s;
+      if constexpr (!FftTypes<T>::kFixed) fft_stage_33<T, true>(sm, ly, pl, s);
+    } else {
+      fft_stage<T, true>(sm, ly, pl, s, 1, meta);
+    }
     __syncthreads();
   }
 }
 
 // ==== compile-time line length ============================================================
-// The same stage sequence as the host plan (radix 3 stages first, then 8, 4, 2; DIT order),
-// known at compile time so that every index, trip count and table offset folds to a constant.
+// The same stage sequence as the host plan (radices 8, 4, 2, then 3; DIT order), known at compile
+// time so that every index, trip count and table offset folds to a constant.  With the radix-3
+// stages outermost the inner spans are powers of two, for which the swizzle (smap) is free of
+// bank conflicts; with them innermost a 192-point stage took 1.8 shared-memory wavefronts for one.
 struct StagePlan {
   int S;
   int R[FFT_MAX_STAGES];
@@ -337,7 +435,7 @@ struct StagePlan {
 __host__ __device__ constexpr StagePlan stage_plan(int N) {
   StagePlan p{};
   int rem = N, s = 0, ns = 1;
-  const int radices[4] = {3, 8, 4, 2};
+  const int radices[4] = {8, 4, 2, 3};
   for (int k = 0; k < 4; ++k) {
     const int R = radices[k];
     while (rem % R == 0 && rem > 1) {
@@ -457,6 +555,131 @@ template <typename T, int N, int LW>
 __device__ __forceinline__ void fft_dit_ct(cpx<T> *sm, int Lc, int lw, const typename FftTypes<T>::Tw *tw,
                                             const unsigned long long *meta = nullptr) {
   ct_dit_from<T, N, LW, 0>(sm, Lc, lw, tw, meta);
+}
+
+// ---- stages between registers and a caller's memory --------------------------------------
+// One stage (RB = 1), or two adjacent stages in registers: the outer one of radix RA over spans
+// NS RB and the inner one of radix RB over span NS, on the RA RB elements e0 + r NS of one thread.
+// The operations and their order are those of the stages one by one; each stage merged, and each
+// end of a transform that reads or writes the caller's memory, saves a round trip through
+// shared memory and a barrier.  ld(lc, e, w) and st(lc, e, w, value) access element e of line
+// (lc, w).
+template <typename T, int R>
+__device__ __forceinline__ void dft_r(cpx<T> *v, typename FftTypes<T>::Dir dir) {
+  if constexpr (R == 8) dft8(v, dir);
+  else if constexpr (R == 4) dft4(v, dir);
+  else if constexpr (R == 3) dft3(v, dir);
+  else if constexpr (R == 2) dft2(v);
+}
+
+// twiddles of one butterfly: before the DFT of an inverse stage (conjugate), after that of a
+// forward one.  All from the table: products of two of them (load_twiddles) put the error of a
+// 192-point apply at 3.2e-7 against 2.7e-7.
+template <typename T, bool INV, int R>
+__device__ __forceinline__ void twiddle_r(cpx<T> (&v)[R], const typename FftTypes<T>::Tw *__restrict__ tw, int jt) {
+#pragma unroll
+  for (int r = 1; r < R; ++r) v[r] = INV ? cmul_conj(v[r], tw[r * jt]) : cmul(v[r], tw[r * jt]);
+}
+
+template <typename T, bool INV, int RA, int RB, int NS, int N, typename LD, typename ST>
+__device__ __forceinline__ void ct_stage_io(int Lc, int lw, const cpx<T> *__restrict__ tw, LD ld, ST st) {
+  constexpr int R = RA * RB;
+  constexpr int NB = N / R;
+  constexpr int TWB = N / (NS * RB);  // table steps of the inner and the outer stage
+  constexpr int TWA = N / (NS * R);
+  const int tot = (Lc * NB) << lw;
+  const T dir = INV ? (T)1 : (T)-1;
+  for (int b = threadIdx.x; b < tot; b += blockDim.x) {
+    const int w = b & ((1 << lw) - 1);
+    const int rest = b >> lw;
+    const int lc = rest / NB;
+    const int q = rest - lc * NB;
+    const int g = q / NS, j = q - g * NS;
+    const int e0 = g * NS * R + j;
+    cpx<T> v[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) v[r] = ld(lc, e0 + r * NS, w);
+    auto outer = [&]() {
+#pragma unroll
+      for (int r2 = 0; r2 < RB; ++r2) {
+        cpx<T> u[RA];
+#pragma unroll
+        for (int k = 0; k < RA; ++k) u[k] = v[r2 + k * RB];
+        if constexpr (INV && NS * RB > 1) twiddle_r<T, true, RA>(u, tw, (j + r2 * NS) * TWA);
+        dft_r<T, RA>(u, dir);
+        if constexpr (!INV && NS * RB > 1) twiddle_r<T, false, RA>(u, tw, (j + r2 * NS) * TWA);
+#pragma unroll
+        for (int k = 0; k < RA; ++k) v[r2 + k * RB] = u[k];
+      }
+    };
+    auto inner = [&]() {
+      if constexpr (RB > 1) {
+#pragma unroll
+        for (int k = 0; k < RA; ++k) {
+          cpx<T> u[RB];
+#pragma unroll
+          for (int r2 = 0; r2 < RB; ++r2) u[r2] = v[k * RB + r2];
+          if constexpr (INV && NS > 1) twiddle_r<T, true, RB>(u, tw, j * TWB);
+          dft_r<T, RB>(u, dir);
+          if constexpr (!INV && NS > 1) twiddle_r<T, false, RB>(u, tw, j * TWB);
+#pragma unroll
+          for (int r2 = 0; r2 < RB; ++r2) v[k * RB + r2] = u[r2];
+        }
+      }
+    };
+    if constexpr (INV) {
+      inner();
+      outer();
+    } else {
+      outer();
+      inner();
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) st(lc, e0 + r * NS, w, v[r]);
+  }
+}
+
+// Stages of the plan of N run in one step from stage hi downwards (forward) or up to stage hi
+// (inverse): two where their radices multiply to at most 16, else one.
+__host__ __device__ constexpr int stages_below(int N, int hi) {
+  const StagePlan p = stage_plan(N);
+  return hi >= 1 && p.R[hi] * p.R[hi - 1] <= 16 ? 2 : 1;
+}
+
+// Forward stages hi..0: the first step reads through ld, the last one writes through st, the steps
+// between them go through shared memory sm(lc, e, w); each step but the last ends in a barrier.
+template <typename T, int N, int HI, typename LD, typename SM, typename ST>
+__device__ __forceinline__ void ct_dif_io(int Lc, int lw, const cpx<T> *tw, LD ld, SM sm, ST st) {
+  constexpr StagePlan P = stage_plan(N);
+  constexpr int C = stages_below(N, HI), LO = HI - C + 1;
+  constexpr int RB = C == 2 ? P.R[LO] : 1;
+  if constexpr (LO == 0) {
+    ct_stage_io<T, false, P.R[HI], RB, 1, N>(Lc, lw, tw, ld, st);
+  } else {
+    auto put = [&](int lc, int e, int w, cpx<T> v) { sm(lc, e, w) = v; };
+    auto get = [&](int lc, int e, int w) { return sm(lc, e, w); };
+    ct_stage_io<T, false, P.R[HI], RB, P.Ns[LO], N>(Lc, lw, tw, ld, put);
+    __syncthreads();
+    ct_dif_io<T, N, LO - 1>(Lc, lw, tw, get, sm, st);
+  }
+}
+// Inverse stages 0..HI of a plan of S stages, in the steps of ct_dif_io in reverse order.
+template <typename T, int N, int HI, int S, typename LD, typename SM, typename ST>
+__device__ __forceinline__ void ct_dit_io(int Lc, int lw, const cpx<T> *tw, LD ld, SM sm, ST st) {
+  constexpr StagePlan P = stage_plan(N);
+  constexpr int C = stages_below(N, HI), LO = HI - C + 1;
+  constexpr int RB = C == 2 ? P.R[LO] : 1;
+  auto put = [&](int lc, int e, int w, cpx<T> v) { sm(lc, e, w) = v; };
+  auto get = [&](int lc, int e, int w) { return sm(lc, e, w); };
+  if constexpr (LO > 0) {
+    ct_dit_io<T, N, LO - 1, S>(Lc, lw, tw, ld, sm, put);
+    __syncthreads();
+    if constexpr (HI == S - 1) ct_stage_io<T, true, P.R[HI], RB, P.Ns[LO], N>(Lc, lw, tw, get, st);
+    else ct_stage_io<T, true, P.R[HI], RB, P.Ns[LO], N>(Lc, lw, tw, get, put);
+  } else {
+    if constexpr (HI == S - 1) ct_stage_io<T, true, P.R[HI], RB, P.Ns[LO], N>(Lc, lw, tw, ld, st);
+    else ct_stage_io<T, true, P.R[HI], RB, P.Ns[LO], N>(Lc, lw, tw, ld, put);
+  }
 }
 
 // Digit reversal of the compile-time plan of N: position -> sample / frequency index (rev)

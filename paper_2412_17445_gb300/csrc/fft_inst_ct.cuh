@@ -1,5 +1,5 @@
 // Explicit instantiations of the apply passes for the compile-time line length RVE_NL.
-// 2D (m = 3) at every length; 3D (m = 6) at the lengths of the 3D grids (<= 128).  RVE_NL is a
+// 2D (m = 3) at every length; 3D (m = 6) at the lengths of the 3D grids (<= 192).  RVE_NL is a
 // multiple of 16 (the shared-memory swizzle of fft.cuh permutes within aligned groups of 16).
 // (2D runs only the fused column pass, mode 1.)
 #define INST_CT2(T)                                                                  \
@@ -39,7 +39,7 @@ template __global__ void k_col_fused2d<RVE_NL, 512 / RVE_NL>(const __grid_consta
 #endif
 #endif
 INST_CT2(double)
-#if RVE_NL <= 128
+#if RVE_NL <= 192
 INST_CT3(float)
 INST_CT3(double)
 #endif

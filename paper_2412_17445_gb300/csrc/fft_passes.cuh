@@ -211,7 +211,7 @@ __device__ __forceinline__ cpx<T> line_value(cpx<T> z, const unsigned long long 
 
 // Transforms of Lc 2^lw lines in shared memory; float64 lines enter as float64 and leave as
 // fixed point (read through line_value).
-template <typename T, int NL, bool INV, int LW>
+template <typename T, int NL, bool INV, int LW, bool MERGE = false>
 __device__ __forceinline__ void fft_lines(cpx<T> *sm, int Lc, int lw, const FftPlan &pl) {
   constexpr bool fixed = sizeof(T) == 8;
   const int Np = line_slots<NL>(pl.Np);
@@ -226,8 +226,21 @@ __device__ __forceinline__ void fft_lines(cpx<T> *sm, int Lc, int lw, const FftP
   cpx<V> *lines = reinterpret_cast<cpx<V> *>(sm);
   if constexpr (NL > 0) {
     const auto *tw = (const typename FftTypes<V>::Tw *)pl.tw;
-    if constexpr (INV) fft_dit_ct<V, NL, LW>(lines, Lc, lw, tw, meta);
-    else fft_dif_ct<V, NL, LW>(lines, Lc, lw, tw, meta);
+    if constexpr (INV && MERGE) {
+      // float32 x-inverse pass in 3D: adjacent small stages merged (ct_stage_io).  In 2D the 20
+      // registers more cost resident blocks (four 512^2: 72.5 us against 70), the forward passes
+      // have none left for it.
+      constexpr int S = stage_plan(NL).S;
+      auto smr = [&](int lc, int e, int) -> cpx<V> & { return lines[lc * NL + smap<NL>(e)]; };
+      auto get = [&](int lc, int e, int w) { return smr(lc, e, w); };
+      auto put = [&](int lc, int e, int w, cpx<V> v) { smr(lc, e, w) = v; };
+      ct_dit_io<V, NL, S - 1, S>(Lc, 0, tw, get, smr, put);
+      __syncthreads();
+    } else if constexpr (INV) {
+      fft_dit_ct<V, NL, LW>(lines, Lc, lw, tw, meta);
+    } else {
+      fft_dif_ct<V, NL, LW>(lines, Lc, lw, tw, meta);
+    }
   } else {
     // lw > 0: consecutive threads take consecutive lines (contiguous addresses); lw = 0: the
     // lines are Np apart, a multiple of the bank count for power-of-two N, so consecutive
@@ -297,31 +310,52 @@ __device__ __forceinline__ void xfwd_tail(cpx<T> *sm, int c, int P, int row0, co
     return;
   }
   const int tot = c * P * hx;
-  for (int i = threadIdx.x; i < tot; i += blockDim.x) {
-    const int l = NL > 0 ? i / (NL / 2 + 1) : (int)fdiv(i, dhx);
-    const int k = i - l * hx;
-    const int ch = (int)fdiv(l, dP), pr = l - ch * P;
-    const cpx<T> zk = sm[l * Np + smap<NL>(pl.unrev[k])];
-    const cpx<T> zn = sm[l * Np + smap<NL>(pl.unrev[k == 0 ? 0 : nx - k])];
-    cpx<T> A, B;
-    if constexpr (sizeof(T) == 8) {
-      // halves of sums of integers
-      const long long kx = __double_as_longlong(zk.x) >> 1, ky = __double_as_longlong(zk.y) >> 1;
-      const long long mx = __double_as_longlong(zn.x) >> 1, my = __double_as_longlong(zn.y) >> 1;
-      A = line_value<T>({__longlong_as_double(kx + mx), __longlong_as_double(ky - my)}, meta, l);
-      B = line_value<T>({__longlong_as_double(ky + my), __longlong_as_double(mx - kx)}, meta, l);
-    } else {
-      A = {(zk.x + zn.x) * (T)0.5, (zk.y - zn.y) * (T)0.5};
-      B = {(zk.y + zn.y) * (T)0.5, (zn.x - zk.x) * (T)0.5};
+  // the positions and values of U entries are read before the first is stored (a store to the
+  // scratch would hold back the table reads of the next entry)
+  constexpr int U = sizeof(T) == 4 ? 4 : 2;
+  for (int base = 0; base < tot; base += U * (int)blockDim.x) {
+    cpx<T> zk[U], zn[U];
+    int pk[U], pn[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int i = min(base + u * (int)blockDim.x + (int)threadIdx.x, tot - 1);
+      const int l = NL > 0 ? i / (NL / 2 + 1) : (int)fdiv(i, dhx);
+      const int k = i - l * hx;
+      pk[u] = l * Np + smap<NL>(__ldg(pl.unrev + k));
+      pn[u] = l * Np + smap<NL>(__ldg(pl.unrev + (k == 0 ? 0 : nx - k)));
     }
-    const int r0 = row0 + 2 * pr, r1 = r0 + 1;
-    if (r0 < g.rows) spec[ch * cs + r0 * hx + k] = A;
-    if (r1 < g.rows) spec[ch * cs + r1 * hx + k] = B;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      zk[u] = sm[pk[u]];
+      zn[u] = sm[pn[u]];
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int i = base + u * (int)blockDim.x + (int)threadIdx.x;
+      if (i >= tot) break;
+      const int l = NL > 0 ? i / (NL / 2 + 1) : (int)fdiv(i, dhx);
+      const int k = i - l * hx;
+      const int ch = (int)fdiv(l, dP), pr = l - ch * P;
+      cpx<T> A, B;
+      if constexpr (sizeof(T) == 8) {
+        // halves of sums of integers
+        const long long kx = __double_as_longlong(zk[u].x) >> 1, ky = __double_as_longlong(zk[u].y) >> 1;
+        const long long mx = __double_as_longlong(zn[u].x) >> 1, my = __double_as_longlong(zn[u].y) >> 1;
+        A = line_value<T>({__longlong_as_double(kx + mx), __longlong_as_double(ky - my)}, meta, l);
+        B = line_value<T>({__longlong_as_double(ky + my), __longlong_as_double(mx - kx)}, meta, l);
+      } else {
+        A = {(zk[u].x + zn[u].x) * (T)0.5, (zk[u].y - zn[u].y) * (T)0.5};
+        B = {(zk[u].y + zn[u].y) * (T)0.5, (zn[u].x - zk[u].x) * (T)0.5};
+      }
+      const int r0 = row0 + 2 * pr, r1 = r0 + 1;
+      if (r0 < g.rows) spec[ch * cs + r0 * hx + k] = A;
+      if (r1 < g.rows) spec[ch * cs + r1 * hx + k] = B;
+    }
   }
 }
 
 // ---- x-inverse head: load row pairs of half spectra, rebuild full lines, DIT inverse ----
-template <typename T, int NL>
+template <typename T, int NL, bool MERGE = false>
 __device__ __forceinline__ void xinv_head(cpx<T> *sm, int c, int P, int row0, const Geo &g, const FftPlan &pl,
                           const cpx<T> *spec, int tr = 0) {
   const int nx = NL > 0 ? NL : g.nx, hx = nx / 2 + 1, Np = line_slots<NL>(pl.Np);
@@ -392,22 +426,41 @@ __device__ __forceinline__ void xinv_head(cpx<T> *sm, int c, int P, int row0, co
       }
     }
   }
-  for (int i = threadIdx.x; i < (tr ? 0 : tot); i += blockDim.x) {
-    const int l = NL > 0 ? i / (NL / 2 + 1) : (int)fdiv(i, dhx);
-    const int k = i - l * hx;
-    const int ch = (int)fdiv(l, dP), pr = l - ch * P;
-    const int r0 = row0 + 2 * pr, r1 = r0 + 1;
-    cpx<T> A = {0, 0}, B = {0, 0};
-    if (r0 < g.rows) A = spec[ch * cs + r0 * hx + k];
-    if (r1 < g.rows) B = spec[ch * cs + r1 * hx + k];
-    if (k == 0 || 2 * k == nx) {
-      A.y = 0;
-      B.y = 0;
+  // as above, U entries' loads before the first shared-memory write
+  constexpr int U = MERGE || NL == 0 ? 4 : 2;
+  for (int base = 0; base < (sizeof(T) == 4 && tr ? 0 : tot); base += U * (int)blockDim.x) {
+    cpx<T> qa[U], qb[U];
+    int pk[U], pn[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int i = base + u * (int)blockDim.x + (int)threadIdx.x;
+      qa[u] = {0, 0};
+      qb[u] = {0, 0};
+      pk[u] = pn[u] = -1;
+      if (i >= tot) continue;
+      const int l = NL > 0 ? i / (NL / 2 + 1) : (int)fdiv(i, dhx);
+      const int k = i - l * hx;
+      const int ch = (int)fdiv(l, dP), pr = l - ch * P;
+      const int r0 = row0 + 2 * pr, r1 = r0 + 1;
+      if (r0 < g.rows) qa[u] = spec[ch * cs + r0 * hx + k];
+      if (r1 < g.rows) qb[u] = spec[ch * cs + r1 * hx + k];
+      pk[u] = l * Np + smap<NL>(__ldg(pl.unrev + k));
+      if (k > 0 && 2 * k < nx) {
+        pn[u] = l * Np + smap<NL>(__ldg(pl.unrev + nx - k));
+      } else {
+        qa[u].y = 0;
+        qb[u].y = 0;
+      }
     }
-    sm[l * Np + smap<NL>(pl.unrev[k])] = {A.x - B.y, A.y + B.x};
-    if (k > 0 && 2 * k < nx) sm[l * Np + smap<NL>(pl.unrev[nx - k])] = {A.x + B.y, B.x - A.y};
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (pk[u] < 0) continue;
+      const cpx<T> A = qa[u], B = qb[u];
+      sm[pk[u]] = {A.x - B.y, A.y + B.x};
+      if (pn[u] >= 0) sm[pn[u]] = {A.x + B.y, B.x - A.y};
+    }
   }
-  fft_lines<T, NL, true, 0>(sm, c * P, 0, pl);
+  fft_lines<T, NL, true, 0, MERGE>(sm, c * P, 0, pl);
 }
 
 }  // namespace
@@ -503,15 +556,16 @@ __device__ __forceinline__ void pro_compute(const ApplyArgs<T> &a, int n, int v,
   wdp += in.w * dpm;
 }
 
-// float32: at least 4 resident blocks per SM (64 registers per thread)
-#ifndef XFWD_MIN_BLOCKS_F32
-#define XFWD_MIN_BLOCKS_F32 4
-#endif
+// float32: 64 registers per thread, 1024 resident threads an SM; 2D blocks have 256 or 512 threads
+// (row_threads)
+template <typename T, int M>
+constexpr int kRowThreads = sizeof(T) == 4 && M == 3 ? 512 : 256;
 // PC > 0 / MODE >= 0: row pairs per block and prologue mode fixed at compile time (the
 // float32 2D passes of the Krylov chunks), so every loop bound and branch folds; PC = 0 /
 // MODE = -1 read them from the launch.
 template <typename T, int M, int NL, int PC, int MODE>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? XFWD_MIN_BLOCKS_F32 : 1) k_xfwd_apply(const __grid_constant__ ApplyGroup<T> grp, FftPlan pl, int P_rt) {
+__global__ void __launch_bounds__(kRowThreads<T, M>, sizeof(T) == 4 ? 1024 / kRowThreads<T, M> : 1) k_xfwd_apply(const __grid_constant__ ApplyGroup<T> grp, FftPlan pl, int P_rt) {
+  pdl_begin();
   const ApplyArgs<T> &a = grp.m[blockIdx.y];
   const int P = PC > 0 ? PC : P_rt;
   const int pm = MODE >= 0 ? MODE : a.pro_mode;
@@ -654,7 +708,8 @@ __device__ __forceinline__ void epi_compute(const ApplyArgs<T> &a, int n, int v,
 }
 
 template <typename T, int M, int NL, int PC, int MODE>
-__global__ void __launch_bounds__(256) k_xinv_apply(const __grid_constant__ ApplyGroup<T> grp, FftPlan pl, int P_rt) {
+__global__ void __launch_bounds__(kRowThreads<T, M>, sizeof(T) == 4 ? 1024 / kRowThreads<T, M> : 1) k_xinv_apply(const __grid_constant__ ApplyGroup<T> grp, FftPlan pl, int P_rt) {
+  pdl_begin();
   const ApplyArgs<T> &a = grp.m[blockIdx.y];
   const int P = PC > 0 ? PC : P_rt;
   const int em = MODE >= 0 ? MODE : a.epi_mode;
@@ -681,7 +736,7 @@ __global__ void __launch_bounds__(256) k_xinv_apply(const __grid_constant__ Appl
   const int n = (int)g.n;
   const int row0 = blk * 2 * P;
   const FDiv dnx = make_fdiv(nx);
-  xinv_head<T, NL>(sm, c, P, row0, g, pl, a.spec, a.tr);
+  xinv_head<T, NL, sizeof(T) == 4 && M == 6>(sm, c, P, row0, g, pl, a.spec, a.tr);
   [[maybe_unused]] const unsigned long long *meta = nullptr;
   if constexpr (sizeof(T) == 8) meta = fx_meta(sm, c * P, 0, Np);
   T d[5] = {0, 0, 0, 0, 0};  // per-thread and warp sums in T, block and grid sums in float64
@@ -692,8 +747,10 @@ __global__ void __launch_bounds__(256) k_xinv_apply(const __grid_constant__ Appl
     const bool ok0 = r0 < g.rows, ok1 = r0 + 1 < g.rows;
     const int v0 = r0 * nx + x, v1 = v0 + nx;
     EpiIn<T, M> in0, in1;
-    if (ok0) epi_load<T, M>(a, n, v0, in0, em);
-    if (ok1) epi_load<T, M>(a, n, v1, in1, em);
+    if (M == 3 || sizeof(T) == 8) {
+      if (ok0) epi_load<T, M>(a, n, v0, in0, em);
+      if (ok1) epi_load<T, M>(a, n, v1, in1, em);
+    }
     const int px = smap<NL>(x);
     T y0[M + 1], y1[M + 1];
 #pragma unroll
@@ -702,8 +759,20 @@ __global__ void __launch_bounds__(256) k_xinv_apply(const __grid_constant__ Appl
       y0[k] = z.x;
       y1[k] = z.y;
     }
-    if (ok0) epi_compute<T, M>(a, n, v0, y0, in0, d, em);
-    if (ok1) epi_compute<T, M>(a, n, v1, y1, in1, d, em);
+    if (M == 3 || sizeof(T) == 8) {
+      if (ok0) epi_compute<T, M>(a, n, v0, y0, in0, d, em);
+      if (ok1) epi_compute<T, M>(a, n, v1, y1, in1, d, em);
+    } else {
+      // 3D float32: one voxel after the other, within the 64 registers of four resident blocks
+      if (ok0) {
+        epi_load<T, M>(a, n, v0, in0, em);
+        epi_compute<T, M>(a, n, v0, y0, in0, d, em);
+      }
+      if (ok1) {
+        epi_load<T, M>(a, n, v1, in0, em);
+        epi_compute<T, M>(a, n, v1, y1, in0, d, em);
+      }
+    }
   }
   if (em == 6) {
     block_partials_k<T, 5>(d, a.part + G, G, blk);
@@ -724,11 +793,53 @@ __global__ void __launch_bounds__(256) k_xinv_apply(const __grid_constant__ Appl
 
 // =========================== column passes (y, z) ============================================
 
+// The spectral multiply on transformed lines in shared memory, in place: projection of the strain
+// channels, |xi|^2 on the phase field (float64 lines: fixed point in, float64 out).
+template <typename T, int M, int NL>
+__device__ __forceinline__ void project_columns(const ColArgs<T> &a, cpx<T> *sm, const unsigned long long *meta, int N,
+                                                int Np, int kx0, int other) {
+  const int lw = a.lw, W = a.W;
+  constexpr int D = (M == 3) ? 2 : 3;
+  const int ky_other = (D == 3) ? a.yplan.rev[other] : 0;
+  for (int i = threadIdx.x; i < (N << lw); i += blockDim.x) {
+    const int p = i >> lw;
+    const int w = i & (W - 1);
+    if (kx0 + w > a.g.hx - 1) continue;
+    int k[3];
+    k[0] = kx0 + w;
+    if (D == 2) {
+      k[1] = a.plan.rev[p];
+    } else {
+      k[1] = ky_other;
+      k[2] = a.plan.rev[p];
+    }
+    ProjDir<T, D> pd;
+    T xi2;
+    willot_dir<T, D>(a.tab, k, a.inv_n, pd, xi2);
+    const int pp = smap<NL>(p);
+    T re[M], im[M];
+#pragma unroll
+    for (int ch = 0; ch < M; ++ch) {
+      const cpx<T> z = line_value<T>(sm[((ch * Np + pp) << lw) + w], meta, (ch << lw) + w);
+      re[ch] = z.x;
+      im[ch] = z.y;
+    }
+    project_mandel<T, M>(re, pd);
+    project_mandel<T, M>(im, pd);
+#pragma unroll
+    for (int ch = 0; ch < M; ++ch) sm[((ch * Np + pp) << lw) + w] = {re[ch], im[ch]};
+    const cpx<T> zp = line_value<T>(sm[((M * Np + pp) << lw) + w], meta, (M << lw) + w);
+    const T sc = xi2 * a.inv_n;
+    sm[((M * Np + pp) << lw) + w] = {zp.x * sc, zp.y * sc};
+  }
+}
+
 // MODE 0: forward only (DIF, result stays digit-reversed along the axis)
 // MODE 1: forward, spectral multiply, inverse (the last axis)
 // MODE 2: inverse only (input digit-reversed along the axis, DIT)
 template <typename T, int M, int MODE, int NL>
 __global__ void __launch_bounds__(256) k_col(const __grid_constant__ ColGroup<T> grp) {
+  pdl_begin();
   const ColArgs<T> &a = grp.base;
   cpx<T> *const spec = grp.spec[blockIdx.z];
   const KrylovScalars *const ks = grp.ks[blockIdx.z];
@@ -751,6 +862,37 @@ __global__ void __launch_bounds__(256) k_col(const __grid_constant__ ColGroup<T>
   }
   const int cs = g.rows * g.hx;
   const int tot = (c * N) << lw;
+  // float32 lines of a compiled length: the first step of the transform reads the scratch into
+  // registers and the last one writes it from them (ct_dif_io, ct_dit_io); a 128-point pass
+  // goes once through shared memory (four times in mode 1) instead of four (eight) times.
+  // 128^3: forward 43 -> 27 us, fused z pass 69 -> 50 us
+  if constexpr (sizeof(T) == 4 && NL > 0) {
+    constexpr int S = stage_plan(NL).S;
+    const cpx<T> *tw = (const cpx<T> *)a.plan.tw;
+    cpx<T> *const col = spec + base_o + kx0;
+    const int wmax = g.hx - kx0;  // columns of the block within the half spectrum
+    auto gld = [&](int lc, int e, int w) -> cpx<T> {
+      return w < wmax ? col[lc * cs + e * es_g + w] : cpx<T>{0, 0};
+    };
+    auto gst = [&](int lc, int e, int w, cpx<T> v) {
+      if (w < wmax) col[lc * cs + e * es_g + w] = v;
+    };
+    auto smr = [&](int lc, int e, int w) -> cpx<T> & { return sm[((lc * NL + smap<NL>(e)) << lw) + w]; };
+    auto sget = [&](int lc, int e, int w) { return smr(lc, e, w); };
+    auto sput = [&](int lc, int e, int w, cpx<T> v) { smr(lc, e, w) = v; };
+    if constexpr (MODE == 0) {
+      ct_dif_io<T, NL, S - 1>(c, lw, tw, gld, smr, gst);
+    } else if constexpr (MODE == 2) {
+      ct_dit_io<T, NL, S - 1, S>(c, lw, tw, gld, smr, gst);
+    } else {
+      ct_dif_io<T, NL, S - 1>(c, lw, tw, gld, smr, sput);
+      __syncthreads();
+      project_columns<T, M, NL>(a, sm, nullptr, N, Np, kx0, other);
+      __syncthreads();
+      ct_dit_io<T, NL, S - 1, S>(c, lw, tw, sget, smr, gst);
+    }
+    return;
+  }
   const FDiv dN = make_fdiv(N);
   // the block's lines are strided in the scratch (one L2 round trip per element): each thread
   // issues KU loads before its first shared-memory store, so they are in flight together
@@ -780,41 +922,7 @@ __global__ void __launch_bounds__(256) k_col(const __grid_constant__ ColGroup<T>
   [[maybe_unused]] const unsigned long long *meta = nullptr;
   if constexpr (sizeof(T) == 8) meta = fx_meta(sm, c, lw, Np);
   if (MODE == 0 || MODE == 1) fft_lines<T, NL, false, -1>(sm, c, lw, a.plan);
-  if (MODE == 1) {
-    constexpr int D = (M == 3) ? 2 : 3;
-    const int ky_other = (D == 3) ? a.yplan.rev[other] : 0;
-    for (int i = threadIdx.x; i < (N << lw); i += blockDim.x) {
-      const int p = i >> lw;
-      const int w = i & (W - 1);
-      if (kx0 + w >= g.hx) continue;
-      int k[3];
-      k[0] = kx0 + w;
-      if (D == 2) {
-        k[1] = a.plan.rev[p];
-      } else {
-        k[1] = ky_other;
-        k[2] = a.plan.rev[p];
-      }
-      ProjDir<T, D> pd;
-      T xi2;
-      willot_dir<T, D>(a.tab, k, a.inv_n, pd, xi2);
-      const int pp = smap<NL>(p);
-      T re[M], im[M];
-#pragma unroll
-      for (int ch = 0; ch < M; ++ch) {
-        const cpx<T> z = line_value<T>(sm[((ch * Np + pp) << lw) + w], meta, (ch << lw) + w);
-        re[ch] = z.x;
-        im[ch] = z.y;
-      }
-      project_mandel<T, M>(re, pd);
-      project_mandel<T, M>(im, pd);
-#pragma unroll
-      for (int ch = 0; ch < M; ++ch) sm[((ch * Np + pp) << lw) + w] = {re[ch], im[ch]};
-      const cpx<T> zp = line_value<T>(sm[((M * Np + pp) << lw) + w], meta, (M << lw) + w);
-      const T sc = xi2 * a.inv_n;
-      sm[((M * Np + pp) << lw) + w] = {zp.x * sc, zp.y * sc};
-    }
-  }
+  if (MODE == 1) project_columns<T, M, NL>(a, sm, meta, N, Np, kx0, other);
   if (MODE == 1 || MODE == 2) fft_lines<T, NL, true, -1>(sm, c, lw, a.plan);
   for (int i = threadIdx.x; i < tot; i += blockDim.x) {
     const int iw = i >> lw;
@@ -844,6 +952,7 @@ __global__ void __launch_bounds__(256) k_col(const __grid_constant__ ColGroup<T>
 // arithmetic as k_col mode 1.
 template <int N, int KC>
 __global__ void __launch_bounds__(1024) k_col_fused2d(const __grid_constant__ ColGroup<float> grp) {
+  pdl_begin();
   const ColArgs<float> &a = grp.base;
   cpx<float> *const spec = grp.spec[blockIdx.y];
   const KrylovScalars *const ks = grp.ks[blockIdx.y];

@@ -106,6 +106,7 @@ static RowKernel<T> row_kernel(int N, int P = 0, int mode = -1) {
         case 256: RS(256); break;
         case 384: RS(384); break;
         case 512: RS(512); break;
+        case 768: RS(768); break;
         case 1024: RS(1024); break;
         default: break;
       }
@@ -119,14 +120,15 @@ static RowKernel<T> row_kernel(int N, int P = 0, int mode = -1) {
     case 64: RK(64);
     case 96: RK(96);
     case 128: RK(128);
+    case 192: RK(192);
     default: break;
   }
   if constexpr (M == 3) {
     switch (N) {
-      case 192: RK(192);
       case 256: RK(256);
       case 384: RK(384);
       case 512: RK(512);
+      case 768: RK(768);
       case 1024: RK(1024);
       default: break;
     }
@@ -163,14 +165,15 @@ static ColKernel<T> col_kernel(int N) {
     case 64: return k_col<T, M, MODE, 64>;
     case 96: return k_col<T, M, MODE, 96>;
     case 128: return k_col<T, M, MODE, 128>;
+    case 192: return k_col<T, M, MODE, 192>;
     default: break;
   }
   if constexpr (M == 3) {
     switch (N) {
-      case 192: return k_col<T, M, MODE, 192>;
       case 256: return k_col<T, M, MODE, 256>;
       case 384: return k_col<T, M, MODE, 384>;
       case 512: return k_col<T, M, MODE, 512>;
+      case 768: return k_col<T, M, MODE, 768>;
       case 1024: return k_col<T, M, MODE, 1024>;
       default: break;
     }
@@ -363,10 +366,10 @@ static FDiv host_fdiv(unsigned d) {
 }
 
 // Radix plans of a line length N = 2^a 3^b, stages in DIT order (stage 0 has span 1):
-//   variant 0: radix-3 stages, then radix 8 as often as possible, then one 4 or 2 (the plan
+//   variant 0: radix 8 as often as possible, one 4 or 2, then radix-3 stages (the plan
 //              of the compile-time kernels, stage_plan in fft.cuh);
 //   variant 1: the radices of variant 0 in reverse order;
-//   variant 2: radix-3 stages, then radix 4 as often as possible, then one 2;
+//   variant 2: radix 4 as often as possible, one 2, then radix-3 stages;
 //   variant 3: the radices of variant 2 in reverse order.
 // The autotuner picks among them for line lengths that run the runtime-length kernels.
 constexpr int kPlanVariants = 4;
@@ -374,10 +377,6 @@ static bool factorize(int N, FftPlan &pl, int variant = 0) {
   if (N < 1 || N > 4096) return false;
   int rem = N;
   std::vector<int> R;
-  while (rem % 3 == 0) {
-    R.push_back(3);
-    rem /= 3;
-  }
   if (variant < 2) {
     while (rem % 8 == 0) {
       R.push_back(8);
@@ -391,6 +390,10 @@ static bool factorize(int N, FftPlan &pl, int variant = 0) {
   while (rem % 2 == 0) {
     R.push_back(2);
     rem /= 2;
+  }
+  while (rem % 3 == 0) {
+    R.push_back(3);
+    rem /= 3;
   }
   if (rem != 1) return false;
   if (variant == 1 || variant == 3) std::reverse(R.begin(), R.end());
@@ -510,10 +513,10 @@ static int ct_len(const rve *h, int a) {
   return h->pvar[a] == 0 ? N : 0;
 }
 
-// lengths with compile-time pass kernels (kernels_fft_<N>.cu): 2D all nine, 3D up to 128
+// lengths with compile-time pass kernels (kernels_fft_<N>.cu): 2D all ten, 3D up to 192
 static bool has_ct_kernel(int N, int m) {
-  static const int ct[9] = {48, 64, 96, 128, 192, 256, 384, 512, 1024};
-  const int cnt = m == 3 ? 9 : 4;
+  static const int ct[10] = {48, 64, 96, 128, 192, 256, 384, 512, 768, 1024};
+  const int cnt = m == 3 ? 10 : 5;
   for (int i = 0; i < cnt; ++i)
     if (ct[i] == N) return true;
   return false;
@@ -592,7 +595,17 @@ static void pass_geometry(const Geo &g, int es, int Preq, int Wreq, int &P, int 
                           size_t &smx, size_t &smy, size_t &smz) {
   const size_t budget = 120 * 1024;
   const int npx = padded(g.nx);
-  P = Preq > 0 ? Preq : (int)(1024 / g.nx);
+  // Default tiles of the float64 passes: the fixed-point stages are chains of 500 instructions that
+  // need resident warps, so blocks are kept to 48 KB (x) and 32 KB (columns) of lines and their
+  // number above two an SM.  Linearisation + apply at (P, W) = (2, 2), the former default at 512^2:
+  // 271 us, at (1, 1): 239 us; at 96^3 (10, 8), likewise: 1815 us, (1, 1): 1681 us, (4, 2): 1526 us.
+  constexpr int kBlocks = 304;
+  if (es == 8 && Preq <= 0) {
+    P = (int)pow2_floor(g.nx < 128 ? 1024 / g.nx : 8);
+    while (P > 1 && ((size_t)g.c * P * npx * 16 > 48 * 1024 || (g.rows + 2 * P - 1) / (2 * P) < kBlocks)) P /= 2;
+  } else {
+    P = Preq > 0 ? Preq : (int)(1024 / g.nx);
+  }
   if (P < 1) P = 1;
   while (P > 1 && (size_t)g.c * P * npx * 2 * es > budget) P /= 2;
   if (2 * P > g.rows + 1) P = (g.rows + 1) / 2;
@@ -603,9 +616,13 @@ static void pass_geometry(const Geo &g, int es, int Preq, int Wreq, int &P, int 
   smx = (size_t)g.c * P * (npx * 2 * es + st);
   auto colW = [&](int N) {
     size_t per = (size_t)g.c * padded(N) * 2 * es;  // one column, all channels, complex
-    size_t w = Wreq > 0 ? (size_t)Wreq : budget / per;
+    size_t w = Wreq > 0 ? (size_t)Wreq : (es == 8 ? 32 * 1024 : budget) / per;
     if (w < 1) w = 1;
     w = pow2_floor(w);
+    if (es == 8 && Wreq <= 0) {
+      const size_t others = (size_t)(g.rows / N);
+      while (w > 1 && (g.hx + w - 1) / w * others < (size_t)kBlocks) w /= 2;
+    }
     if (w > 16) w = 16;
     while (w > 1 && per * w > budget) w /= 2;
     while (w > 1 && w / 2 >= (size_t)g.hx) w /= 2;
@@ -639,8 +656,8 @@ static int set_smem_attrs(rve *h, size_t need) {
   }
   if (done_dev == dev) return RVE_OK;
 #define SA(...) TRY(set_one_attr(h, (const void *)(__VA_ARGS__), optin))
-  static const int kAllCt[9] = {48, 64, 96, 128, 192, 256, 384, 512, 1024};  // kernels_fft_<N>.cu
-  for (int li = -1; li < 9; ++li) {
+  static const int kAllCt[10] = {48, 64, 96, 128, 192, 256, 384, 512, 768, 1024};  // kernels_fft_<N>.cu
+  for (int li = -1; li < 10; ++li) {
     const int N = li < 0 ? 0 : kAllCt[li];
     const bool pow2 = (N & (N - 1)) == 0;
     SA((row_kernel<float, 3, true>(N))); SA((row_kernel<float, 3, false>(N)));
@@ -666,6 +683,36 @@ static int set_smem_attrs(rve *h, size_t need) {
 #undef SA
   done_dev = dev;
   return RVE_OK;
+}
+
+// Threads of an x-pass block: 512 for a float32 2D block of 1024 voxel pairs.  One 512^2 RVE has less
+// than one such block an SM, and its passes are chains of loads and stages: 33.5 us an apply with
+// 256 threads, 30.7 us with 512.
+template <typename T, int M>
+static int row_threads(int P, int nx) {
+  return sizeof(T) == 4 && M == 3 && P * nx >= 1024 ? 512 : 256;
+}
+
+// Launch with a programmatic dependency on the kernel before (pdl; the kernel starts with
+// pdl_begin) or an ordinary one.  The later passes of a float32 operator apply take it: their blocks
+// are resident when the pass before ends (243 x 729: 43.2 -> 40.9 us, 128^3: 243 -> 237 us).  Not
+// the float64 ones (512^2: 98 us without, 106 us with it: blocks that wait where there is room
+// leave the SMs unevenly loaded) nor the BiCGStab chunks (64^2 float64 increment: 23 -> 27.5 ms).
+template <typename... KA, typename... A>
+static void launch(bool pdl, void (*k)(KA...), dim3 grid, int block, size_t smem, cudaStream_t st, const A &...args) {
+  cudaLaunchConfig_t cfg;
+  memset((void *)&cfg, 0, sizeof cfg);
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at;
+  memset((void *)&at, 0, sizeof at);
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = pdl ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, k, args...);  // errors: the caller's CKL
 }
 
 // ---- typed launch helpers ----------------------------------------------------------------
@@ -705,7 +752,7 @@ static int spec_tr(const rve *h) {
 // nm RVEs of h's shape (scratch spec[i], Krylov scalars ks[i]) as one launch per pass
 template <typename T, int M>
 static int launch_columns_n(rve *h, cpx<T> *const *spec, const KrylovScalars *const *ks, int nm, int Wy,
-                            int Wz, size_t smy, size_t smz, cudaStream_t st) {
+                            int Wz, size_t smy, size_t smz, cudaStream_t st, bool pdl = false) {
   ColGroup<T> G;
   memset((void *)&G, 0, sizeof G);
   ColArgs<T> &ca = G.base;
@@ -735,8 +782,8 @@ static int launch_columns_n(rve *h, cpx<T> *const *spec, const KrylovScalars *co
     const int v = Wy >= 4 ? 2 : (Wy >= 2 ? 1 : 0);
     const int kc = fused_cols(g.ny, v);
     dim3 grid((g.hx + kc - 1) / kc, nm);
-    fused_col_kernel(g.ny, v)<<<grid, kc * g.ny / 2, fused_col_smem(g.ny, v), st>>>(
-        *reinterpret_cast<ColGroup<float> *>(&G));
+    launch(pdl, fused_col_kernel(g.ny, v), grid, kc * g.ny / 2, fused_col_smem(g.ny, v), st,
+           *reinterpret_cast<ColGroup<float> *>(&G));
     h->launches += 1;
   } else if (g.nz == 1) {
     ca.axis = 1;
@@ -744,7 +791,7 @@ static int launch_columns_n(rve *h, cpx<T> *const *spec, const KrylovScalars *co
     ca.lw = log2i(Wy);
     ca.plan = plan_of<T>(h, 1);
     dim3 grid((g.hx + Wy - 1) / Wy, 1, nm);
-    col_kernel<T, M, 1>(ct_len(h, 1))<<<grid, 256, smy, st>>>(G);
+    launch(pdl, col_kernel<T, M, 1>(ct_len(h, 1)), grid, 256, smy, st, G);
     h->launches += 1;
   } else {
     ca.axis = 1;
@@ -752,18 +799,18 @@ static int launch_columns_n(rve *h, cpx<T> *const *spec, const KrylovScalars *co
     ca.lw = log2i(Wy);
     ca.plan = plan_of<T>(h, 1);
     dim3 gy((g.hx + Wy - 1) / Wy, g.nz, nm);
-    col_kernel<T, M, 0>(ct_len(h, 1))<<<gy, 256, smy, st>>>(G);
+    launch(pdl, col_kernel<T, M, 0>(ct_len(h, 1)), gy, 256, smy, st, G);
     ca.axis = 2;
     ca.W = Wz;
     ca.lw = log2i(Wz);
     ca.plan = plan_of<T>(h, 2);
     dim3 gz((g.hx + Wz - 1) / Wz, g.ny, nm);
-    col_kernel<T, M, 1>(ct_len(h, 2))<<<gz, 256, smz, st>>>(G);
+    launch(pdl, col_kernel<T, M, 1>(ct_len(h, 2)), gz, 256, smz, st, G);
     ca.axis = 1;
     ca.W = Wy;
     ca.lw = log2i(Wy);
     ca.plan = plan_of<T>(h, 1);
-    col_kernel<T, M, 2>(ct_len(h, 1))<<<gy, 256, smy, st>>>(G);
+    launch(pdl, col_kernel<T, M, 2>(ct_len(h, 1)), gy, 256, smy, st, G);
     h->launches += 3;
   }
   CKL();
@@ -772,8 +819,8 @@ static int launch_columns_n(rve *h, cpx<T> *const *spec, const KrylovScalars *co
 
 template <typename T, int M>
 static int launch_columns(rve *h, cpx<T> *spec, const KrylovScalars *ks, int Wy, int Wz, size_t smy,
-                          size_t smz) {
-  return launch_columns_n<T, M>(h, &spec, &ks, 1, Wy, Wz, smy, smz, h->stream);
+                          size_t smz, bool pdl = false) {
+  return launch_columns_n<T, M>(h, &spec, &ks, 1, Wy, Wz, smy, smz, h->stream, pdl);
 }
 
 // ---- the scaled operator apply y = S J x ------------------------------------------------
@@ -834,13 +881,14 @@ static int apply_scaled(rve *h, TK *x, const double *xE_ptr, TK *y, int pro_mode
   const int P = dbl ? h->Px_d : h->Px;
   const int Gx = dbl ? h->Gx_d : h->Gx;
   const size_t smx = dbl ? h->smx_d : h->smx_k;
-  row_kernel<TK, M, true>(ct_len(h, 0), P, a.pro_mode)<<<Gx, 256, smx, h->stream>>>(solo(a), plan_of<TK>(h, 0), P);
+  row_kernel<TK, M, true>(ct_len(h, 0), P, a.pro_mode)<<<Gx, row_threads<TK, M>(P, h->g.nx), smx, h->stream>>>(solo(a), plan_of<TK>(h, 0), P);
   h->launches += 1;
   CKL();
   TRY((launch_columns<TK, M>(h, a.spec, ks, dbl ? h->Wy_d : h->Wy, dbl ? h->Wz_d : h->Wz,
-                             dbl ? h->smy_d : h->smy_k, dbl ? h->smz_d : h->smz_k)));
+                             dbl ? h->smy_d : h->smy_k, dbl ? h->smz_d : h->smz_k, !dbl)));
   // fin 3, 4: one more block for the E slot
-  row_kernel<TK, M, false>(ct_len(h, 0), P, a.epi_mode)<<<Gx + (yE ? 1 : 0), 256, smx, h->stream>>>(solo(a), plan_of<TK>(h, 0), P);
+  launch(!dbl, row_kernel<TK, M, false>(ct_len(h, 0), P, a.epi_mode), dim3(Gx + (yE ? 1 : 0)),
+         row_threads<TK, M>(P, h->g.nx), smx, h->stream, solo(a), plan_of<TK>(h, 0), P);
   h->launches += 1;
   CKL();
   return RVE_OK;
@@ -1324,14 +1372,15 @@ static int issue_chunk_n(rve *const *mem, int nm, cudaStream_t st) {
   const dim3 gx(Gx, nm), gpw(h->Gpw, nm);
   const int Wy = dbl ? h->Wy_d : h->Wy, Wz = dbl ? h->Wz_d : h->Wz;
   const size_t smy = dbl ? h->smy_d : h->smy_k, smz = dbl ? h->smz_d : h->smz_k;
+  const int tx = row_threads<TK, M>(P, h->g.nx);
   for (int j = 0; j < krylov_chunk_len(); ++j) {
-    row_kernel<TK, M, true>(ct_len(h, 0), P, merged ? 5 : 1)<<<gx, 256, smx, st>>>(A1, plx, P);
+    row_kernel<TK, M, true>(ct_len(h, 0), P, merged ? 5 : 1)<<<gx, tx, smx, st>>>(A1, plx, P);
     TRY((launch_columns_n<TK, M>(h, spec, ksc, nm, Wy, Wz, smy, smz, st)));
-    row_kernel<TK, M, false>(ct_len(h, 0), P, 1)<<<gx, 256, smx, st>>>(A1, plx, P);  // + alpha
-    row_kernel<TK, M, true>(ct_len(h, 0), P, 2)<<<gx, 256, smx, st>>>(A2, plx, P);
+    row_kernel<TK, M, false>(ct_len(h, 0), P, 1)<<<gx, tx, smx, st>>>(A1, plx, P);  // + alpha
+    row_kernel<TK, M, true>(ct_len(h, 0), P, 2)<<<gx, tx, smx, st>>>(A2, plx, P);
     TRY((launch_columns_n<TK, M>(h, spec, ksc, nm, Wy, Wz, smy, smz, st)));
     // + omega (merged: + convergence, the x / r update left pending)
-    row_kernel<TK, M, false>(ct_len(h, 0), P, merged ? 6 : 2)<<<gx, 256, smx, st>>>(A2, plx, P);
+    row_kernel<TK, M, false>(ct_len(h, 0), P, merged ? 6 : 2)<<<gx, tx, smx, st>>>(A2, plx, P);
     if (!merged) k_kxr<TK><<<gpw, 256, 0, st>>>(K);                          // + convergence
     h->launches += merged ? 4 : 5;
     CKL();
@@ -1559,11 +1608,11 @@ static int project_step_f32_t(rve *h) {
   a.pro_mode = 4;
   a.epi_mode = 3;
   a.tr = spec_tr<float, M>(h);
-  row_kernel<float, M, true>(ct_len(h, 0), h->Px, a.pro_mode)<<<h->Gx, 256, h->smx_k, h->stream>>>(solo(a), plan_of<float>(h, 0), h->Px);
+  row_kernel<float, M, true>(ct_len(h, 0), h->Px, a.pro_mode)<<<h->Gx, row_threads<float, M>(h->Px, h->g.nx), h->smx_k, h->stream>>>(solo(a), plan_of<float>(h, 0), h->Px);
   h->launches += 1;
   CKL();
   TRY((launch_columns<float, M>(h, a.spec, nullptr, h->Wy, h->Wz, h->smy_k, h->smz_k)));
-  row_kernel<float, M, false>(ct_len(h, 0), h->Px, a.epi_mode)<<<h->Gx, 256, h->smx_k, h->stream>>>(solo(a), plan_of<float>(h, 0), h->Px);
+  row_kernel<float, M, false>(ct_len(h, 0), h->Px, a.epi_mode)<<<h->Gx, row_threads<float, M>(h->Px, h->g.nx), h->smx_k, h->stream>>>(solo(a), plan_of<float>(h, 0), h->Px);
   h->launches += 1;
   CKL();
   return RVE_OK;
@@ -1664,10 +1713,14 @@ static int autotune_t(rve *h) {
   // some boxes.  Float32 2D grids of at least 256 x 256 therefore take P = 2 and W = 4
   // untimed; narrower rows (where larger P fills a block) are tuned.
   const bool fix_p2 = sizeof(TK) == 4 && h->g.d == 2 && h->g.rows >= 256 && h->g.nx >= 256;
+  // Float64 2D grids of up to two row pairs an SM take P = W = 1 untimed: 64^2 31.9 us an apply against
+  // 32.8 to 43, 512^2 98 us against 108 to 119, differences that the short timing missed.
+  const bool fix_11 = sizeof(TK) == 8 && h->g.d == 2 && h->g.rows <= 608;
   for (int pi = 0; pi < 4; ++pi)
     for (int wi = 0; wi < 5; ++wi) {
       int P, Gx, Wy, Wz;
       size_t smx, smy, smz;
+      if (fix_11 && (pi || wi)) continue;
       if (fix_p2 && (Ps[pi] != 2 || Ws[wi] != 4)) continue;
       pass_geometry(h->g, es, Ps[pi], Ws[wi], P, Gx, Wy, Wz, smx, smy, smz);
       // clamped: covered by another candidate (the fixed schedule takes its clamped form)
@@ -2924,13 +2977,14 @@ static int apply_batch_t(rve *const *hs, int n, const void *const *x, const doub
     ks[i] = nullptr;
   }
   const dim3 gx(Gx, n);
-  row_kernel<TK, M, true>(ct_len(h, 0), P, A.m[0].pro_mode)<<<gx, 256, smx, st>>>(A, plan_of<TK>(h, 0), P);
+  row_kernel<TK, M, true>(ct_len(h, 0), P, A.m[0].pro_mode)<<<gx, row_threads<TK, M>(P, h->g.nx), smx, st>>>(A, plan_of<TK>(h, 0), P);
   h->launches += 1;
   CKL();
   TRY((launch_columns_n<TK, M>(h, spec, ks, n, dbl ? h->Wy_d : h->Wy, dbl ? h->Wz_d : h->Wz,
-                               dbl ? h->smy_d : h->smy_k, dbl ? h->smz_d : h->smz_k, st)));
+                               dbl ? h->smy_d : h->smy_k, dbl ? h->smz_d : h->smz_k, st, !dbl)));
   const dim3 gi(Gx + 1, n);  // one more block a member for the E slot
-  row_kernel<TK, M, false>(ct_len(h, 0), P, A.m[0].epi_mode)<<<gi, 256, smx, st>>>(A, plan_of<TK>(h, 0), P);
+  launch(!dbl, row_kernel<TK, M, false>(ct_len(h, 0), P, A.m[0].epi_mode), gi, row_threads<TK, M>(P, h->g.nx), smx,
+         st, A, plan_of<TK>(h, 0), P);
   h->launches += 1;
   CKL();
   return RVE_OK;

@@ -202,13 +202,14 @@ __device__ __forceinline__ void block_partials_k(const TK (&v)[NQ], double *part
     }
     __syncthreads();
     const int nw = (blockDim.x + 31) >> 5;
-    if (NQ <= 4 && nw <= 8) {
-      // one warp, eight lanes a quantity: three dependent float64 adds
+    constexpr int LQ = NQ <= 2 ? 16 : 8;  // lanes a quantity
+    if (NQ <= 4 && nw <= LQ) {
+      // one warp: three or four dependent float64 adds
       if (threadIdx.x < 32) {
-        const int q = threadIdx.x >> 3, w = threadIdx.x & 7;
+        const int q = threadIdx.x / LQ, w = threadIdx.x % LQ;
         double sum = q < NQ && w < nw ? red[w][q] : 0.0;
 #pragma unroll
-        for (int o = 4; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+        for (int o = LQ / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
         if (w == 0 && q < NQ) part[q * G + blk] = sum;
       }
     } else if (threadIdx.x < NQ) {
@@ -243,6 +244,14 @@ __device__ __forceinline__ void block_max_partials(double (&v)[NQ], double *part
     }
   }
   __syncthreads();
+}
+
+// Programmatic dependent launch, at the top of the passes of an apply: wait for the kernels before
+// (at once where the launch has no such dependency), then let the next pass's blocks take free SM
+// resources, where they wait in turn.
+__device__ __forceinline__ void pdl_begin() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // ---- kernel argument structs ------------------------------------------------------------
