@@ -72,8 +72,26 @@ __host__ __device__ __forceinline__ long long fx_from_bits(unsigned long long b,
   return (long long)b < 0 ? -r : r;
 }
 
-// v 2^e as float64 bits, rounded to nearest, ties to even; saturates to infinity, and
-// flushes results below the normal range to zero
+// magnitude of a result outside the normal range, from its 64 leading bits m and biased exponent less
+// one be (fx_to_bits): a subnormal number in units of 2^-1074 (a full last unit carries into the
+// normal range), zero or infinity.  Kept out of line: it would cost the loops that store the lines
+// registers.
+#ifdef __CUDA_ARCH__
+static __noinline__ __device__
+#else
+static inline
+#endif
+unsigned long long fx_end_bits(unsigned long long m, int be) {
+  if (be > 0) return 0x7FF0000000000000ull;
+  const int sh = 11 - be;
+  if (sh > 64) return 0ull;
+  const unsigned long long q = sh < 64 ? m >> sh : 0ull;
+  const unsigned long long rest = m << (64 - sh);  // against a half, 2^63
+  return q + (rest > 0x8000000000000000ull || (rest == 0x8000000000000000ull && (q & 1u)) ? 1ull : 0ull);
+}
+
+// v 2^e as float64 bits, rounded once to nearest, ties to even, also into the subnormal range;
+// infinity from the midpoint above the largest finite number on
 __host__ __device__ __forceinline__ unsigned long long fx_to_bits(long long v, int e) {
   const unsigned long long sign = (unsigned long long)v & 0x8000000000000000ull;
   unsigned long long m = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
@@ -85,8 +103,7 @@ __host__ __device__ __forceinline__ unsigned long long fx_to_bits(long long v, i
 #endif
   m <<= lz;
   const int be = e + 63 - lz + 1022;  // biased exponent less one: the leading bit adds it back
-  if (be < 0) return sign;
-  if (be > 2044) return sign | 0x7FF0000000000000ull;
+  if ((unsigned)be > 2045u) return sign | fx_end_bits(m, be);
   const unsigned long long q = m >> 11;
   const unsigned long long rest = m & 2047u;
   const unsigned long long up = rest + (q & 1u) > 1024u ? 1ull : 0ull;

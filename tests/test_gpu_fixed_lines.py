@@ -80,3 +80,20 @@ def test_shared_exponent(shape):
         z[g.n // 3] = bad
         assert np.all(np.isnan(_apply(g, z, 0.25)[:g.m * g.n]))
     g.close()
+
+
+@pytest.mark.parametrize("shape", [(48, 64), (27, 81), (16, 12, 6)])
+def test_subnormal_results(shape):
+    """Operands far below the normal range (2^-1040) give the scaled result of the operands at unit
+    magnitude, off by the subnormal roundings alone: about three units of 2^-1074 an entry after
+    the projection, which carries the factor 1 / n, times sqrt(n) through the two inverse transforms
+    of the RMS (the roundings before the projection and in the last pass are smaller by sqrt(n))."""
+    _, g, _ = _setup(shape, 21)
+    rng = np.random.default_rng(7)
+    k = 1040
+    small = np.ldexp(rng.standard_normal((g.m + 1) * g.n), -k)  # rounded to the subnormal grid
+    want = _apply(g, np.ldexp(small, k), 0.25)
+    got = np.ldexp(_apply(g, small, np.ldexp(0.25, -k)), k)
+    err = np.sqrt(np.mean((got - want).reshape(g.m + 1, -1) ** 2, axis=1))
+    assert np.all(err <= 4.0 * np.sqrt(g.n) * 2.0 ** (k - 1074)), err
+    g.close()
