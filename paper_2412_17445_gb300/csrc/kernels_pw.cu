@@ -52,12 +52,22 @@ __device__ __forceinline__ void eig2(const double *e, double *z, double *Q) {
   Q[4] = ct;
 }
 
+// The exponent field that a magnitude would have if the field went below 1, and x 2^(1023 - ex) in
+// float32 for a subnormal x and such an exponent.  Out of line: strains below 2^-1022 are rare.
+__device__ __noinline__ int exponent_of_subnormal(double x) {
+  return 12 - __clzll(__double_as_longlong(x) & 0xFFFFFFFFFFFFFll);
+}
+__device__ __noinline__ float scaled_subnormal(double x, int ex) {
+  const float m = (float)(__double_as_longlong(x) & 0xFFFFFFFFFFFFFll);
+  return copysignf(ldexpf(m, -51 - ex), (float)__double2hiint(x));
+}
+
 // x 2^(1023 - ex) in float32 for the biased exponent ex of a magnitude of x's matrix: the bits of
 // x, truncated, so that no conversion goes through the float64 pipe
 __device__ __forceinline__ float scaled_f32(double x, int ex) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
   const int eb = (int)(b >> 52 & 2047), e = eb - ex + 127;
-  if (eb == 0 || e <= 0) return 0.f;
+  if (eb == 0 || e <= 0) return eb == 0 && ex < 128 && x != 0.0 ? scaled_subnormal(x, ex) : 0.f;
   return __uint_as_float((unsigned)(b >> 32) & 0x80000000u | (unsigned)min(e, 255) << 23 |
                          (unsigned)(b >> 29) & 0x7FFFFFu);
 }
@@ -153,7 +163,8 @@ __device__ __forceinline__ void jacobi_f64(double (&A)[6], double *Q, int ex) {
 // pipe takes a warp instruction every 16 cycles).
 __device__ __forceinline__ void eig3(const double *e, double *z, double *Q) {
   const double scale = fabs(e[0]) + fabs(e[4]) + fabs(e[8]) + fabs(e[1]) + fabs(e[2]) + fabs(e[5]);
-  const int ex = (int)((unsigned long long)__double_as_longlong(scale) >> 52);
+  int ex = (int)((unsigned long long)__double_as_longlong(scale) >> 52);
+  if (ex == 0) ex = exponent_of_subnormal(scale);
   float Af[6] = {scaled_f32(e[0], ex), scaled_f32(e[4], ex), scaled_f32(e[8], ex),
                  scaled_f32(e[5], ex), scaled_f32(e[2], ex), scaled_f32(e[1], ex)};
   float q[4] = {1.f, 0.f, 0.f, 0.f};
@@ -265,7 +276,7 @@ __global__ void __launch_bounds__(256) k_constitutive(ConstArgs a, TK *tan) {
         for (int i = 0; i < D; ++i) {
           zp[i] = pos_part(z[i]);
           ws[i] = mu2 * zp[i];
-          wg[i] = __double2hiint(zp[i]) != 0 ? g * ws[i] : mu2 * neg_part(z[i]);
+          wg[i] = __double_as_longlong(zp[i]) != 0 ? g * ws[i] : mu2 * neg_part(z[i]);
         }
       };
       if constexpr (D == 2) {
@@ -355,7 +366,7 @@ __global__ void __launch_bounds__(256) k_constitutive(ConstArgs a, TK *tan) {
       const double tie = 1e-12 * zmax;
 #pragma unroll
       for (int i = 0; i < D; ++i) {
-        Lt[i * 4] = __double2hiint(zp[i]) != 0 ? (TK)1 : (TK)0;
+        Lt[i * 4] = __double_as_longlong(zp[i]) != 0 ? (TK)1 : (TK)0;
 #pragma unroll
         for (int j = i + 1; j < D; ++j) {
           const double d = z[i] - z[j];

@@ -61,3 +61,28 @@ def test_residual_and_tangent(shape, kind):
     assert np.max(np.abs(Je - B.mandel_from_tensor(Jo[0]))) < 1e-11 * np.max(np.abs(Jo[0]))
     assert np.max(np.abs(Jp - Jo[1].reshape(-1))) < 1e-11 * np.max(np.abs(Jo[1]))
     g.close()
+
+
+@pytest.mark.parametrize("k", [1010, 1040])
+def test_residual_of_tiny_strains(k):
+    """The stress is positively homogeneous in the strain: strains at 2^-k, their eigenvectors included,
+    give the residual of the same strains at unit magnitude.  1e-11 of the stress scale as above;
+    near and below 2^-1022 also the subnormal roundings, in units u = 2^-1074: about 2 u a strain
+    entry and as much again in the eigenvalues, times the stiffness, and four u an entry, times sqrt(n),
+    through the transforms of the RMS."""
+    shape = (6, 8, 4)
+    inp = ms.random_rve(shape, 7)
+    _, _, phi, H = ms.random_state(inp, 8)
+    a = np.random.default_rng(4).standard_normal(shape + (3, 3))
+    small = np.ldexp(B.mandel_from_tensor(a + np.swapaxes(a, -1, -2)), -k)
+    stiff = np.max(inp.E * (1 - inp.nu) / ((1 + inp.nu) * (1 - 2 * inp.nu)))
+    g = B.RVE(inp)
+    F = []
+    for eps in (np.ldexp(small, k), small):
+        g.set_state(eps, phi, H, 0.0)
+        g.linearize(B.RVE_CTRL_STRAIN, 0.0)
+        F.append(g.residual()[0])
+    scale = stiff * np.max(np.abs(np.ldexp(small, k)))
+    err = np.sqrt(np.mean((np.ldexp(F[1], k) - F[0]) ** 2))
+    assert err <= 1e-11 * scale + 4 * (np.sqrt(g.n) + 2 * stiff + 2) * 2.0 ** (k - 1074)
+    g.close()
