@@ -726,7 +726,7 @@ __global__ void __launch_bounds__(kRowThreads<T, M>, sizeof(T) == 4 ? 1024 / kRo
     if (a.fin == 4) {
       if (threadIdx.x == 0) *a.yE = *a.xE_ptr;
     } else if (threadIdx.x < 32) {
-      const double sE = warp_sum_exact<false>(a.part, G);
+      const double sE = warp_sum<false>(a.part, G);
       if (threadIdx.x == 0) *a.yE = sE;
     }
     return;
@@ -783,10 +783,8 @@ __global__ void __launch_bounds__(kRowThreads<T, M>, sizeof(T) == 4 ? 1024 / kRo
   if (a.fin == 1 || a.fin == 2 || a.fin == 5 || a.fin == 6) {
     // the member's last block finalises the iteration's scalars (no separate launch)
     if (last_block_arrives(a.arrive, G)) {
-      if (a.fin == 1) fin_alpha<true>(a.ksw, a.part, G);
-      else if (a.fin == 2) fin_omega<true>(a.ksw, a.part, G);
-      else if (a.fin == 5) fin_alpha_clear<true>(a.ksw, a.part, G);
-      else fin_omega_conv<true>(a.ksw, a.part, G);
+      if constexpr (sizeof(T) == 4 && M == 6) finalise_out_of_line(a.fin, a.ksw, a.part, G);
+      else finalise(a.fin, a.ksw, a.part, G);
     }
   }
 }

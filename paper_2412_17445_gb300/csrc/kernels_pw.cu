@@ -486,7 +486,7 @@ __global__ void __launch_bounds__(256) k_constitutive(ConstArgs a, TK *tan) {
 // =========================== reductions ======================================================
 // Every quantity by one warp: exact sums (krylov_fin.cuh) or maxima.
 __device__ __forceinline__ double warp_reduce_partials(const double *p, int G, int is_max) {
-  if (!is_max) return warp_sum_exact<false>(p, G);
+  if (!is_max) return warp_sum<false>(p, G);
   double s = -1e308;
   for (int i = threadIdx.x & 31; i < G; i += 32) s = fmax(s, p[i]);
 #pragma unroll

@@ -6,16 +6,88 @@
 #pragma once
 #include "rve_kern.cuh"
 
-// Exact sum of G float64 partials by one warp, rounded once: each value becomes a 128-bit integer
-// in units of 2^-53 ulp of the largest exponent seen (53 mantissa bits, 53 below them, room for
-// 2^20 terms above), and integers add exactly in any order.  A compensated float64 sum needs five
-// operations a value and seven a tree level on a pipe that takes a warp instruction every 16
-// cycles (the block-wide one took 4.2 us a quantity, 33 us of a 512^2 BiCGStab iteration's
-// seven sums); integer adds run at full rate, a warp a quantity.  Non-finite values fall back
-// to a float64 sum, which propagates them.  CG: the partials were written by other blocks of
-// the running kernel, so they are read past L1 (ld.global.cg).
+// 128-bit integer sum over the lanes of a warp (modulo 2^128)
+__device__ __forceinline__ __int128 warp_add128(__int128 acc) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long lo = __shfl_xor_sync(0xffffffffu, (unsigned long long)acc, o);
+    const unsigned long long hi = __shfl_xor_sync(0xffffffffu, (unsigned long long)((unsigned __int128)acc >> 64), o);
+    acc = (__int128)((unsigned __int128)acc + (((unsigned __int128)hi << 64) | lo));
+  }
+  return acc;
+}
+__device__ __forceinline__ int clz128(unsigned __int128 mag) {
+  const unsigned long long top = (unsigned long long)(mag >> 64);
+  return top ? __clzll(top) : 64 + __clzll((unsigned long long)mag);
+}
+// acc 2^unit as float64, rounded once
+__device__ __forceinline__ double round128(__int128 acc, int unit) {
+  if (acc == 0) return 0.0;
+  const bool neg = acc < 0;
+  unsigned __int128 mag = neg ? (unsigned __int128)(-acc) : (unsigned __int128)acc;
+  const int lz = clz128(mag);
+  mag <<= lz;
+  // the leading 64 bits with the rest as a sticky bit, rounded to 53 once
+  const unsigned long long lead = (unsigned long long)(mag >> 64) | ((unsigned long long)mag ? 1ull : 0ull);
+  const double r = scalbn(__ull2double_rn(lead), 64 - lz + unit);
+  return neg ? -r : r;
+}
+// Significant bits that a sum of G terms needs where bits below its unit were cut: fewer than 2 G + 64
+// units are lost (one a term, one a lane and batch), a sixteenth of the last place of a sum of
+// this many bits.
+__device__ __forceinline__ int bits_needed(int G) { return 57 + 32 - __clz(2 * G + 64); }
+__device__ __forceinline__ int bits_of(__int128 acc) {
+  return 128 - clz128((unsigned __int128)(acc < 0 ? -acc : acc));
+}
+
+// The sum of finite terms that cancel below those bits, from a first window on: with a unit 53 bits
+// below the last place of the largest term nothing overflows; from there the sum is known to 2 G + 64 units,
+// so it fits a window of 128 bits whose unit lies up to 125 bits lower, and what is above the window
+// cancels modulo 2^128.  Repeated until the sum has its bits, or the unit is the last place of the
+// smallest term, where nothing is cut.  Rare, and out of line.
 template <bool CG>
-__device__ __forceinline__ double warp_sum_exact(const double *p, int G) {
+__device__ __noinline__ double warp_sum_cancelled(const double *p, int G) {
+  const int lane = threadIdx.x & 31;
+  int emax = 1, emin = 2046;
+  for (int i = lane; i < G; i += 32) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(CG ? __ldcg(p + i) : p[i]);
+    const int ex = max((int)(b >> 52) & 2047, 1);
+    emax = max(emax, ex);
+    if (b << 1) emin = min(emin, ex);
+  }
+  emax = __reduce_max_sync(0xffffffffu, emax);
+  emin = __reduce_min_sync(0xffffffffu, emin);
+  int unit = emax - 1075 - 53;
+  for (;;) {
+    unsigned __int128 s = 0;
+    for (int i = lane; i < G; i += 32) {
+      const unsigned long long b = (unsigned long long)__double_as_longlong(CG ? __ldcg(p + i) : p[i]);
+      const int ex = (int)(b >> 52) & 2047;
+      const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | (ex ? 1ull << 52 : 0ull);
+      const int sh = (ex ? ex : 1) - 1075 - unit;
+      const unsigned __int128 t =
+          sh >= 0 ? (sh < 128 ? (unsigned __int128)m << sh : 0) : (unsigned __int128)(sh > -64 ? m >> -sh : 0ull);
+      s += (b >> 63) ? 0 - t : t;
+    }
+    const __int128 acc = warp_add128((__int128)s);
+    const int have = bits_of(acc);
+    if (unit <= emin - 1075 || have >= bits_needed(G)) return round128(acc, unit);
+    unit = max(unit - (125 - max(have, 32 - __clz(2 * G + 64))), emin - 1075);
+  }
+}
+
+// Sum of G float64 partials by one warp, to 9/16 of a unit in the last place whatever cancels
+// (rounded once where no bit was cut): each value becomes a 128-bit integer in units of 2^-53 ulp of
+// the largest exponent seen (53 mantissa bits, 53 below them, room for 2^20 terms above), and
+// integers add exactly in any order.  Bits below the unit are cut; if fewer bits of the sum are left
+// than that allows, warp_sum_cancelled takes over.  A compensated float64 sum needs five operations
+// a value and seven a tree level on a pipe that takes a warp instruction every 16 cycles (the
+// block-wide one took 4.2 us a quantity, 33 us of a 512^2 BiCGStab iteration's seven sums); integer
+// adds run at full rate, a warp a quantity.  Non-finite values fall back to a float64 sum, which
+// propagates them.  CG: the partials were written by other blocks of the running kernel, so they
+// are read past L1 (ld.global.cg).
+template <bool CG>
+__device__ __forceinline__ double warp_sum(const double *p, int G) {
   constexpr int U = 8;  // values per lane in flight
   const int lane = threadIdx.x & 31;
   __int128 acc = 0;
@@ -53,22 +125,10 @@ __device__ __forceinline__ double warp_sum_exact(const double *p, int G) {
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     return s;
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const unsigned long long lo = __shfl_xor_sync(0xffffffffu, (unsigned long long)acc, o);
-    const long long hi = __shfl_xor_sync(0xffffffffu, (long long)(acc >> 64), o);
-    acc += (__int128)(((unsigned __int128)(unsigned long long)hi << 64) | lo);
-  }
-  if (acc == 0) return 0.0;
-  const bool neg = acc < 0;
-  unsigned __int128 mag = neg ? (unsigned __int128)(-acc) : (unsigned __int128)acc;
-  const unsigned long long top = (unsigned long long)(mag >> 64);
-  const int lz = top ? __clzll(top) : 64 + __clzll((unsigned long long)mag);
-  mag <<= lz;
-  // the leading 64 bits with the rest as a sticky bit, rounded to 53 once
-  const unsigned long long lead = (unsigned long long)(mag >> 64) | ((unsigned long long)mag ? 1ull : 0ull);
-  const double r = scalbn(__ull2double_rn(lead), 64 - lz + E - 1075 - 53);
-  return neg ? -r : r;
+  acc = warp_add128(acc);
+  // (E <= 54, all zeros among them: the unit is at most 2^-1074 and nothing was cut)
+  if (E > 54 && bits_of(acc) < bits_needed(G)) return warp_sum_cancelled<CG>(p, G);
+  return round128(acc, E - 1075 - 53);
 }
 
 // NQ sums of G partials each (quantity q at part + q G), one warp a quantity; every thread of the
@@ -77,7 +137,7 @@ template <int NQ, bool CG>
 __device__ __forceinline__ void block_sums(const double *part, int G, double (&out)[NQ]) {
   __shared__ double res[NQ];
   for (int q = threadIdx.x >> 5; q < NQ; q += blockDim.x >> 5) {
-    const double s = warp_sum_exact<CG>(part + (size_t)q * G, G);
+    const double s = warp_sum<CG>(part + (size_t)q * G, G);
     if ((threadIdx.x & 31) == 0) res[q] = s;
   }
   __syncthreads();
@@ -245,4 +305,16 @@ __device__ __forceinline__ void fin_omega_conv(KrylovScalars *ks, const double *
     ks->beta_f = (float)ks->beta;
     ks->pE_f = (float)(ks->pE * ks->escale);
   }
+}
+
+// the update of ApplyArgs::fin by the member's last block
+__device__ __forceinline__ void finalise(int fin, KrylovScalars *ks, const double *part, int G) {
+  if (fin == 1) fin_alpha<true>(ks, part, G);
+  else if (fin == 2) fin_omega<true>(ks, part, G);
+  else if (fin == 5) fin_alpha_clear<true>(ks, part, G);
+  else fin_omega_conv<true>(ks, part, G);
+}
+// for the float32 3D x-inverse pass, which with this inlined spills at its 64 registers
+static __device__ __noinline__ void finalise_out_of_line(int fin, KrylovScalars *ks, const double *part, int G) {
+  finalise(fin, ks, part, G);
 }
