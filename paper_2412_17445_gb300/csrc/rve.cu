@@ -588,6 +588,8 @@ static size_t pow2_floor(size_t x) {
 
 static int padded(int N) { return N + (N - 1) / 8; }
 
+constexpr int kSMs = 152;  // of one GB300
+
 // launch geometry of the FFT passes for element size es (bytes of one real value):
 // P row pairs per x-pass block, W kx columns per column-pass block.  P and W come from the
 // tuner (rve_tune) or these defaults.
@@ -599,7 +601,7 @@ static void pass_geometry(const Geo &g, int es, int Preq, int Wreq, int &P, int 
   // need resident warps, so blocks are kept to 48 KB (x) and 32 KB (columns) of lines and their
   // number above two an SM.  Linearisation + apply at (P, W) = (2, 2), the former default at 512^2:
   // 271 us, at (1, 1): 239 us; at 96^3 (10, 8), likewise: 1815 us, (1, 1): 1681 us, (4, 2): 1526 us.
-  constexpr int kBlocks = 304;
+  constexpr int kBlocks = 2 * kSMs;
   if (es == 8 && Preq <= 0) {
     P = (int)pow2_floor(g.nx < 128 ? 1024 / g.nx : 8);
     while (P > 1 && ((size_t)g.c * P * npx * 16 > 48 * 1024 || (g.rows + 2 * P - 1) / (2 * P) < kBlocks)) P /= 2;
@@ -1713,9 +1715,14 @@ static int autotune_t(rve *h) {
   // some boxes.  Float32 2D grids of at least 256 x 256 therefore take P = 2 and W = 4
   // untimed; narrower rows (where larger P fills a block) are tuned.
   const bool fix_p2 = sizeof(TK) == 4 && h->g.d == 2 && h->g.rows >= 256 && h->g.nx >= 256;
-  // Float64 2D grids of up to two row pairs an SM take P = W = 1 untimed: 64^2 31.9 us an apply against
-  // 32.8 to 43, 512^2 98 us against 108 to 119, differences that the short timing missed.
-  const bool fix_11 = sizeof(TK) == 8 && h->g.d == 2 && h->g.rows <= 608;
+  // Float64 2D grids of up to two row pairs an SM and rows of up to 768 points, at most eight times as
+  // long as the columns, take P = W = 1 untimed, since the short timing misses differences of a
+  // few per cent.  Of 14 schedules it was the fastest or within 1 % of it on 16 grids of that
+  // range, 32 x 48 to 576^2, 576 x 16 to 96 x 768 (64^2: 33 us an apply against 33 to 62,
+  // 512^2: 96 us against 104 to 113).  Longer rows are timed: 8 x 2187 takes 201 us at (1, 1) and
+  // 181 us at (2, 4), 48 x 2048 154 and 145 us at (1, 2), 512 x 1024 180 and 175 us at (1, 4).
+  const bool fix_11 = sizeof(TK) == 8 && h->g.d == 2 && h->g.rows <= 4 * kSMs && h->g.nx <= 768 &&
+                      h->g.nx <= 8 * h->g.rows;
   for (int pi = 0; pi < 4; ++pi)
     for (int wi = 0; wi < 5; ++wi) {
       int P, Gx, Wy, Wz;
