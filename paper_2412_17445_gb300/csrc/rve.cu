@@ -687,19 +687,21 @@ static int set_smem_attrs(rve *h, size_t need) {
   return RVE_OK;
 }
 
-// Threads of an x-pass block: 512 for a float32 2D block of 1024 voxel pairs.  One 512^2 RVE has less
-// than one such block an SM, and its passes are chains of loads and stages: 33.5 us an apply with
-// 256 threads, 30.7 us with 512.
+// Threads of an x-pass block: 512 for a float32 2D block of 1024 voxel pairs, whose passes are chains of
+// loads and stages.  An apply with 256 and 512 threads: 512^2 27.9 and 24.8 us, 256 x 1024 41.6 and
+// 33.3, 1296^2 241 and 201; groups of 512^2 RVEs, two 37.2 and 35.2, three 47.8 and 50.5, four 63.4
+// and 64.5, eight 109.6 and 113.9 (from three on there are blocks enough without).
 template <typename T, int M>
 static int row_threads(int P, int nx) {
   return sizeof(T) == 4 && M == 3 && P * nx >= 1024 ? 512 : 256;
 }
 
 // Launch with a programmatic dependency on the kernel before (pdl; the kernel starts with
-// pdl_begin) or an ordinary one.  The later passes of a float32 operator apply take it: their blocks
-// are resident when the pass before ends (243 x 729: 43.2 -> 40.9 us, 128^3: 243 -> 237 us).  Not
-// the float64 ones (512^2: 98 us without, 106 us with it: blocks that wait where there is room
-// leave the SMs unevenly loaded) nor the BiCGStab chunks (64^2 float64 increment: 23 -> 27.5 ms).
+// pdl_begin, rve_kern.cuh) or an ordinary one.  The later passes of a float32 operator apply take it, which
+// hides their launch behind the pass before (tuned, against ordinary launches: 64^2 14.9 -> 11.0 us,
+// 243 x 729 39.5 -> 35.3, 128^3 241 -> 230).  The float64 passes and the BiCGStab chunks take
+// ordinary launches; they were measured only with blocks triggered early (512^2 98 -> 106 us, 64^2
+// float64 increment 23 -> 27.5 ms).
 template <typename... KA, typename... A>
 static void launch(bool pdl, void (*k)(KA...), dim3 grid, int block, size_t smem, cudaStream_t st, const A &...args) {
   cudaLaunchConfig_t cfg;

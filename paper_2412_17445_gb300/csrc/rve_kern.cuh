@@ -247,11 +247,13 @@ __device__ __forceinline__ void block_max_partials(double (&v)[NQ], double *part
 }
 
 // Programmatic dependent launch, at the top of the passes of an apply: wait for the kernels before
-// (at once where the launch has no such dependency), then let the next pass's blocks take free SM
-// resources, where they wait in turn.
+// (at once where the launch has no such dependency).  No pass triggers its successor early: the
+// successor's launch is prepared while the pass runs and takes place when its last block ends, on
+// an empty GPU.  Triggered at the top of the pass instead, the next blocks settle wherever an SM has
+// room while the pass still runs, several to one SM and none to others (float32 2048 x 256:
+// 62 us an apply, 123 us with the early trigger, 68 us with ordinary launches; 512^2: 24.5, 30.7, 29).
 __device__ __forceinline__ void pdl_begin() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // ---- kernel argument structs ------------------------------------------------------------
