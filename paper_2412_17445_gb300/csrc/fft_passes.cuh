@@ -783,8 +783,7 @@ __global__ void __launch_bounds__(kRowThreads<T, M>, sizeof(T) == 4 ? 1024 / kRo
   if (a.fin == 1 || a.fin == 2 || a.fin == 5 || a.fin == 6) {
     // the member's last block finalises the iteration's scalars (no separate launch)
     if (last_block_arrives(a.arrive, G)) {
-      if constexpr (sizeof(T) == 4 && M == 6) finalise_out_of_line(a.fin, a.ksw, a.part, G);
-      else finalise(a.fin, a.ksw, a.part, G);
+      finalise(a.fin, a.ksw, a.part, G);
     }
   }
 }

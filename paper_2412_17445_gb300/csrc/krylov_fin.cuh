@@ -20,35 +20,28 @@ __device__ __forceinline__ int clz128(unsigned __int128 mag) {
   const unsigned long long top = (unsigned long long)(mag >> 64);
   return top ? __clzll(top) : 64 + __clzll((unsigned long long)mag);
 }
-// acc 2^unit as float64, rounded once
-__device__ __forceinline__ double round128(__int128 acc, int unit) {
-  if (acc == 0) return 0.0;
-  const bool neg = acc < 0;
-  unsigned __int128 mag = neg ? (unsigned __int128)(-acc) : (unsigned __int128)acc;
-  const int lz = clz128(mag);
+// the leading 64 of 128 bits, the rest as a sticky bit (lz leading zeros, below 128)
+__device__ __forceinline__ unsigned long long leading128(unsigned __int128 mag, int lz) {
   mag <<= lz;
-  // the leading 64 bits with the rest as a sticky bit, rounded to 53 once
-  const unsigned long long lead = (unsigned long long)(mag >> 64) | ((unsigned long long)mag ? 1ull : 0ull);
-  const double r = scalbn(__ull2double_rn(lead), 64 - lz + unit);
-  return neg ? -r : r;
+  return (unsigned long long)(mag >> 64) | ((unsigned long long)mag ? 1ull : 0ull);
 }
-// Significant bits that a sum of G terms needs where bits below its unit were cut: fewer than 2 G + 64
-// units are lost (one a term, one a lane and batch), a sixteenth of the last place of a sum of
-// this many bits.
-__device__ __forceinline__ int bits_needed(int G) { return 57 + 32 - __clz(2 * G + 64); }
-__device__ __forceinline__ int bits_of(__int128 acc) {
-  return 128 - clz128((unsigned __int128)(acc < 0 ? -acc : acc));
-}
+// Significant bits that a sum of up to 2^20 terms needs where bits below its unit were cut: fewer than
+// 2 G + 64 units are lost (one a term, one a lane and batch), a sixteenth of the last place of a
+// sum of this many bits.
+constexpr int kSumBits = 79;
 
 // The sum of finite terms that cancel below those bits, from a first window on: with a unit 53 bits
 // below the last place of the largest term nothing overflows; from there the sum is known to 2 G + 64 units,
-// so it fits a window of 128 bits whose unit lies up to 125 bits lower, and what is above the window
+// so it fits a window of 128 bits whose unit lies up to 103 bits lower, and what is above the window
 // cancels modulo 2^128.  Repeated until the sum has its bits, or the unit is the last place of the
-// smallest term, where nothing is cut.  Rare, and out of line.
+// smallest term, where nothing is cut.  Also rounds results outside the normal range.  Rare, and kept short
+// (no unrolling) and out of line: the finalisers are chains of code that run once, and inlined or
+// unrolled this costs a 64^3 BiCGStab iteration 3 to 8 us of 108.
 template <bool CG>
 __device__ __noinline__ double warp_sum_cancelled(const double *p, int G) {
   const int lane = threadIdx.x & 31;
   int emax = 1, emin = 2046;
+#pragma unroll 1
   for (int i = lane; i < G; i += 32) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(CG ? __ldcg(p + i) : p[i]);
     const int ex = max((int)(b >> 52) & 2047, 1);
@@ -58,8 +51,10 @@ __device__ __noinline__ double warp_sum_cancelled(const double *p, int G) {
   emax = __reduce_max_sync(0xffffffffu, emax);
   emin = __reduce_min_sync(0xffffffffu, emin);
   int unit = emax - 1075 - 53;
+#pragma unroll 1
   for (;;) {
     unsigned __int128 s = 0;
+#pragma unroll 1
     for (int i = lane; i < G; i += 32) {
       const unsigned long long b = (unsigned long long)__double_as_longlong(CG ? __ldcg(p + i) : p[i]);
       const int ex = (int)(b >> 52) & 2047;
@@ -70,9 +65,14 @@ __device__ __noinline__ double warp_sum_cancelled(const double *p, int G) {
       s += (b >> 63) ? 0 - t : t;
     }
     const __int128 acc = warp_add128((__int128)s);
-    const int have = bits_of(acc);
-    if (unit <= emin - 1075 || have >= bits_needed(G)) return round128(acc, unit);
-    unit = max(unit - (125 - max(have, 32 - __clz(2 * G + 64))), emin - 1075);
+    const unsigned __int128 mag = (unsigned __int128)(acc < 0 ? -acc : acc);
+    const int lz = clz128(mag);
+    if (acc == 0 && unit <= emin - 1075) return 0.0;
+    if (unit <= emin - 1075 || 128 - lz >= kSumBits) {
+      const double r = scalbn(__ull2double_rn(leading128(mag, lz)), 64 - lz + unit);
+      return acc < 0 ? -r : r;
+    }
+    unit = max(unit - (125 - max(128 - lz, 22)), emin - 1075);
   }
 }
 
@@ -126,9 +126,17 @@ __device__ __forceinline__ double warp_sum(const double *p, int G) {
     return s;
   }
   acc = warp_add128(acc);
-  // (E <= 54, all zeros among them: the unit is at most 2^-1074 and nothing was cut)
-  if (E > 54 && bits_of(acc) < bits_needed(G)) return warp_sum_cancelled<CG>(p, G);
-  return round128(acc, E - 1075 - 53);
+  const unsigned __int128 mag = (unsigned __int128)(acc < 0 ? -acc : acc);
+  const int lz = clz128(mag);
+  // rounded by integers: a conversion and scalbn are a chain on the float64 pipe.  be: biased exponent less
+  // one, as in fx_to_bits; at E <= 54 the unit is at most 2^-1074 and nothing was cut
+  const int be = 64 - lz + (E - 1075 - 53) + 63 + 1022;
+  if (__builtin_expect((128 - lz < kSumBits && E > 54) || (unsigned)be > 2045u, 0))
+    return E == 1 && lz == 128 ? 0.0 : warp_sum_cancelled<CG>(p, G);
+  const unsigned long long lead = leading128(mag, lz);
+  const unsigned long long q = lead >> 11;
+  const unsigned long long b = ((unsigned long long)be << 52) + q + ((lead & 2047u) + (q & 1u) > 1024u ? 1ull : 0ull);
+  return __longlong_as_double((long long)(b | (acc < 0 ? 1ull << 63 : 0ull)));
 }
 
 // NQ sums of G partials each (quantity q at part + q G), one warp a quantity; every thread of the
@@ -313,8 +321,4 @@ __device__ __forceinline__ void finalise(int fin, KrylovScalars *ks, const doubl
   else if (fin == 2) fin_omega<true>(ks, part, G);
   else if (fin == 5) fin_alpha_clear<true>(ks, part, G);
   else fin_omega_conv<true>(ks, part, G);
-}
-// for the float32 3D x-inverse pass, which with this inlined spills at its 64 registers
-static __device__ __noinline__ void finalise_out_of_line(int fin, KrylovScalars *ks, const double *part, int G) {
-  finalise(fin, ks, part, G);
 }
