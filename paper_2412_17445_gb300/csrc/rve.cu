@@ -1707,6 +1707,11 @@ static int autotune_t(rve *h) {
   CK(cudaEventCreate(&e1));
   float best = 1e30f;
   int bP = h->Px, bW = h->Wy;
+  struct Timed {
+    int P, W;
+    float ms;
+  };
+  std::vector<Timed> timed;
   // The candidates are timed as solo applies, but the batched step runs the float32 2D passes
   // of several RVEs concurrently as grouped launches.  On 512^2 composites the step ran at
   // 59.3-59.8 increments/s with P = 1, 63.5-64.1 with P = 2 and 57.7 with P = 4, while the
@@ -1746,12 +1751,25 @@ static int autotune_t(rve *h) {
       CK(cudaEventSynchronize(e1));
       float ms = 0;
       CK(cudaEventElapsedTime(&ms, e0, e1));
+      timed.push_back({P, Wy, ms});
       if (ms < best) {
         best = ms;
         bP = P;
         bW = Wy;
       }
     }
+  // Solo float32 applies of small 3D grids are bound by the latency of their passes, and several tiles tie
+  // to the resolution of this timing, while a group of RVEs fills the GPU and prefers large blocks: of the
+  // candidates within 3 % of the fastest take the most row pairs a block, then the most columns.  Two
+  // 32 x 128 x 32 RVEs take 64, 60, 60 and 54 us an apply at (4, 2), (4, 4), (4, 8) and (8, 8), solo 39.5 to
+  // 40.3; five 18 x 128 x 18 take 87, 70 and 62 us at (2, 4), (4, 4) and (8, 4), solo 33.  Larger grids
+  // take the fastest (two 48 x 108 x 96 156 us, with this rule 160), and so do 2D ones.
+  if (sizeof(TK) == 4 && h->g.d == 3 && h->g.n <= 1 << 17)
+    for (const Timed &c : timed)  // in the order of P, then W
+      if (c.ms <= 1.03f * best) {
+        bP = c.P;
+        bW = c.W;
+      }
   pass_geometry(h->g, es, bP, bW, h->Px, h->Gx, h->Wy, h->Wz, h->smx_k, h->smy_k, h->smz_k);
   if (sizeof(TK) == 8)
     pass_geometry(h->g, 8, bP, bW, h->Px_d, h->Gx_d, h->Wy_d, h->Wz_d, h->smx_d, h->smy_d, h->smz_d);
