@@ -130,7 +130,9 @@ __device__ __forceinline__ void fx_load_lines(cpx<double> *sm, int Lc, int lw, i
   unsigned long long *meta = fx_meta(sm, Lc, lw, Np);
   const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int W = 1 << lw, w = lane & (W - 1);
-  const int spl = Lc < nw ? nw / Lc : 1;  // warps per group
+  // warps per group; one where its lanes take at most four elements of the group each (sharing a group
+  // costs three barriers)
+  const int spl = Lc < nw && (N << lw) > 128 ? nw / Lc : 1;
   const int step = (32 >> lw) * spl;
   const unsigned long long *raw = reinterpret_cast<const unsigned long long *>(sm);
   longlong2 *out = reinterpret_cast<longlong2 *>(sm);
