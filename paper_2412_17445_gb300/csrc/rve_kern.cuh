@@ -101,10 +101,12 @@ __device__ __forceinline__ T ks_scalar(double d, float f) {
 }
 
 // ---- float64 roots and reciprocals ------------------------------------------------------
-// By a float32 seed (22 bits) and one third-order Newton (Halley) correction, which leaves about
-// one unit in the last place: 3 and 5 float64 operations.  The seed's bits are moved by integer
-// instructions, not converted through the float64 pipe.  Arguments whose seed leaves the normal
-// range take the library function.
+// By a float32 seed r, good to 2^-21, and the series of the exact value in its residual h to second
+// order: 1 / x = r / (1 - h) = r (1 + h + h^2 + ...) with h = 1 - x r, and 1 / sqrt(x) = r (1 - h)^-1/2 =
+// r (1 + h / 2 + 3 h^2 / 8 + ...) with h = 1 - x r^2.  What is cut, h^3, is 2^-63, so the reciprocal is
+// within one step of the rounded quotient and the root within one unit in the last place: 3 and 5
+// float64 operations.  The seed's bits are moved by integer instructions, not converted through the
+// float64 pipe.  Arguments whose seed leaves the normal range take the library function.
 __device__ __forceinline__ double f64_of_seed(float r, int shift) {  // r 2^shift, r in [2^-2, 2)
   const unsigned b = __float_as_uint(r);
   return __hiloint2double((int)((b >> 3) + ((896u + (unsigned)shift) << 20)), (int)(b << 29));
