@@ -95,3 +95,33 @@ def test_few_large_column_blocks_spread_over_the_gpu():
         times.append(min(best[1:]))
         g.close()
     assert times[0] < 0.7 * times[1], times
+
+
+def test_tuned_increment_of_768_points():
+    """The two-row-pair, 512-thread passes of 768 points in the modes of a solve: a tuned MIXED increment
+    against the float64 handle's, to the 1e-5 that MIXED is held to."""
+    inp = ms.fibre_composite(n=768, ny=256, radius=12.0, fraction=0.4, notch_len=32, seed=3)
+    steps = []
+    for precision in (B.RVE_MIXED, B.RVE_FP64):
+        g = B.RVE(inp, precision=precision, newton_tol=1e-8, krylov_tol=1e-2)
+        g.startup()
+        steps.append(g.crack_increment(1.0))
+        g.close()
+    m, d = steps
+    assert m["fallbacks"] == 0
+    assert abs(m["E"] - d["E"]) <= 1e-5 * abs(d["E"]) and abs(m["gamma"] - d["gamma"]) <= 1e-5 * abs(d["gamma"])
+    assert np.max(np.abs(np.subtract(m["sigma"], d["sigma"]))) <= 1e-5 * np.max(np.abs(d["sigma"]))
+
+
+@pytest.mark.parametrize("shape", [(256, 768), (18, 768), (6, 8, 4)])
+def test_constraint_row_terms(shape):
+    """The constraint row of a tuned MIXED apply against its terms: each a product of two float32 numbers, a
+    dozen of them and the lanes of a warp summed in float32, ten roundings (6e-7) of the terms' magnitudes."""
+    inp, (eps, E, phi, H), g = _rve(shape, 61)
+    g.autotune()
+    lin = solver.Linearization(solver.problem_from_input(inp), eps, E, phi, H)
+    de, dp, dE = ms.random_direction(inp, 63)
+    _, _, JE = g.apply(B.mandel_from_tensor(de), dp, dE)
+    terms = lin.w * dp
+    assert abs(JE - np.sum(terms)) <= 6e-7 * np.sum(np.abs(terms))
+    g.close()
