@@ -168,7 +168,7 @@ def apply_roofline(torch, B, g, inp, reps=50):
 # (nominal 1.25), 1/64 of its float32 rate
 FP64_TFLOPS = 1.25
 
-APPLY_TRAFFIC = {"sha": "1a8f7543afd5cb90", "bytes": 116208384, "rves": 4}
+APPLY_TRAFFIC = {"sha": "d731f0c3bd1d5433", "bytes": 115584256, "rves": 4}
 APPLY_SOURCES = ["fft.cuh", "fft_passes.cuh", "rve_kern.cuh", "krylov_fin.cuh", "fft_inst_ct.cuh", "kernels_fft_512.cu"]
 
 

@@ -180,7 +180,7 @@ int rve_set_state(rve_t *h, const double *eps_tilde, const double *phi, const do
 /* Autotuner of the FFT passes: times the operator apply (Eq. CrackLength_linearization)
  * on the device for candidate tiles (row pairs per x-pass block, kx columns per y/z-pass
  * block; fixed for float32 2D grids of at least 256 x 256 and float64 2D grids of at most 608
- * rows) and then, for RVE_MIXED handles,
+ * rows of at most 768 points, no longer than eight times the columns) and then, for RVE_MIXED handles,
  * per axis whose length has no compile-time kernel, for candidate radix plans (radix-8 or
  * radix-4 stages, in either order), and keeps the fastest (RVE_FP64 handles keep the default
  * plan, so their rounding does not depend on timings).  Later handles of the same grid and precision in

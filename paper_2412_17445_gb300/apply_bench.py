@@ -1,6 +1,7 @@
 """Operator-apply microbenchmark: time rve_apply_device on a synthetic workload.
 
   python -m paper_2412_17445_gb300.apply_bench --workload composite512 --precision mixed --reps 20 [--batch 4]
+  python -m paper_2412_17445_gb300.apply_bench --workload porous96 --precision mixed --reps 3 --newton
   python -m paper_2412_17445_gb300.apply_bench --workload composite512 --precision mixed --increment
   python -m paper_2412_17445_gb300.apply_bench --workload composite512 --precision mixed --batch-increment 16
 
@@ -26,8 +27,8 @@ def workload(name):
         return ms.fibre_composite(n=512, radius=12.0, fraction=0.4, notch_len=32)
     if name == "panel64":
         return ms.homogeneous_panel(64, notch_len=16)
-    if name == "porous128":
-        return ms.porous_solid(n=128)
+    if name.startswith("porous"):
+        return ms.porous_solid(n=int(name[6:]))
     if name.startswith("panel"):
         n = int(name[5:])
         return ms.homogeneous_panel(n, notch_len=n // 4)
@@ -63,6 +64,8 @@ def main():
     ap.add_argument("--reps", type=int, default=20)
     ap.add_argument("--batch", type=int, default=1,
                     help="RVEs of the workload's shape applied as one group (rve_apply_device_batch)")
+    ap.add_argument("--newton", action="store_true",
+                    help="linearise anew before every apply (constitutive update, residual passes)")
     ap.add_argument("--batch-increment", type=int, default=0,
                     help="instead of applies: this many RVEs of the workload (seeds differ), start-up, one "
                          "warm-up batched increment, then one batched increment between cudaProfilerStart and "
@@ -101,6 +104,9 @@ def main():
     g = gs[0]
 
     def run():
+        if args.newton:
+            for q in gs:
+                q.linearize(B.RVE_CTRL_CRACK, 1.0)
         if args.batch == 1:
             x, xE, y, yE = bufs[0]
             g.apply_device(x.data_ptr(), xE.data_ptr(), y.data_ptr(), yE.data_ptr())

@@ -91,9 +91,11 @@ __device__ __forceinline__ int pad8(int e) { return e + (e >> 3); }
 // Shared-memory slot of element e of a line of compile-time length NL (> 0, a multiple of
 // 16, line bases at multiples of 16): bits 0..3 are XOR-ed with bits 3..6.  Within every
 // half-warp of 8-byte accesses this is conflict-free for unit-stride runs, for the stride-8
-// runs of the span-1 radix-8 stage and for the 64 g + j + 8 r runs of the span-8 stage
-// (checked for every stage of every compiled length), and it needs no padding.  NL = 0
-// keeps the padded layout.
+// runs of the span-1 radix-8 stage and for the 64 g + j + 8 r runs of the span-8 stage, and it
+// needs no padding.  Not for everything: radix-3 stages and the Hermitian gathers of the x passes
+// conflict (192-point float32 x passes 5.0 of 20.7 M wavefronts, 48-point 1.8 of 3.4 M, 128-point
+// 0.5 of 5.2 M), and so do the 16-byte elements of the float64 lines (512 points 0.4 of 1.2 M).
+// NL = 0 keeps the padded layout.
 template <int NL>
 __device__ __forceinline__ int smap(int e) {
   if constexpr (NL > 0) return e ^ ((e >> 3) & 15);
@@ -424,8 +426,9 @@ __device__ void fft_dit(cpx<T> *sm, const LineLayout &ly, const FftPlan &pl, con
 // ==== compile-time line length ============================================================
 // The same stage sequence as the host plan (radices 8, 4, 2, then 3; DIT order), known at compile
 // time so that every index, trip count and table offset folds to a constant.  With the radix-3
-// stages outermost the inner spans are powers of two, for which the swizzle (smap) is free of
-// bank conflicts; with them innermost a 192-point stage took 1.8 shared-memory wavefronts for one.
+// stages outermost the inner spans are powers of two, for which the swizzle (smap) keeps the
+// radix-8 stages free of bank conflicts; with them innermost a 192-point stage took 1.8
+// shared-memory wavefronts for one.
 struct StagePlan {
   int S;
   int R[FFT_MAX_STAGES];

@@ -484,7 +484,7 @@ __global__ void __launch_bounds__(256) k_constitutive(ConstArgs a, TK *tan) {
 }
 
 // =========================== reductions ======================================================
-// Every quantity by one warp: exact sums (krylov_fin.cuh) or maxima.
+// Every quantity by one warp: sums (warp_sum, krylov_fin.cuh) or maxima.
 __device__ __forceinline__ double warp_reduce_partials(const double *p, int G, int is_max) {
   if (!is_max) return warp_sum<false>(p, G);
   double s = -1e308;
